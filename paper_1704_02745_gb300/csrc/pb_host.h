@@ -6,6 +6,7 @@
 
 #include "pb.h"
 #include "pb_internal.cuh"
+#include "resident.cuh"
 #include "setup.cuh"
 #include "solve.cuh"
 
@@ -14,6 +15,7 @@ struct pb_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int num_sms = 1;
+  int max_smem = 0;  // shared memory a CTA may ask for, bytes
   pb::Scal *host_scal = nullptr;  // pinned, for convergence polls
   // pb_ctx_stats counters; a server's internal context counts into its parent's
   std::atomic<unsigned long long> launches{0}, h2d{0}, d2h{0};
@@ -57,6 +59,13 @@ struct pb_grid {
   // cached device graph of `graph_ticks` ticks
   cudaGraphExec_t graph = nullptr;
   int graph_mode = -1, graph_coef = -1, graph_ticks = 0;
+  // resident inner solves (resident.cu): the plan of (res_mode, res_coef), the
+  // packets of the grid-wide sums, the device graph of a whole solve
+  pb::ResPlan res_plan;
+  int res_mode = -1, res_coef = -1;
+  bool res_fits = false;
+  void *res_packets = nullptr;
+  cudaGraphExec_t res_graph = nullptr;
 };
 
 pb_status pb_fail(pb_status s, const std::string &msg);

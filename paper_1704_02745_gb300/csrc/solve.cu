@@ -1401,8 +1401,11 @@ KernelGrid kernel_grid(int mode, int coef, int num_sms, bool single) {
 
 #ifdef PB_FAULT_TEST
 // Test builds only: make the next `count` first-plane stage waits give up at
-// once (see g_fault_abandon_waits).  Returns 0, or PB_ERR_CUDA.
+// once (see g_fault_abandon_waits), and the next `count` first grid-wide sums
+// of the resident solve.  Returns 0, or PB_ERR_CUDA.
+int pb_resident_abandon_sums(int count);  // resident.cu
 extern "C" int pb_test_abandon_waits(int count) {
+  if (pb_resident_abandon_sums(count)) return 3;
   return cudaMemcpyToSymbol(pb::g_fault_abandon_waits, &count, sizeof(int)) == cudaSuccess ? 0 : 3;
 }
 #endif
