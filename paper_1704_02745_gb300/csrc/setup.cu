@@ -6,6 +6,7 @@
 // o + (i + 0.5)*h, and the inside test |m - x_a|^2 < r_a^2 as
 // (dx*dx + dy*dy) + dz*dz, each operation rounded on its own (__d*_rn), so
 // the dielectric map is the same bit pattern whatever the evaluation order.
+#include <type_traits>
 #include <cmath>
 
 #include "pb_internal.cuh"
@@ -188,89 +189,142 @@ __device__ __forceinline__ void ghost_pos(const Geom &g, long t, double &px, dou
 constexpr int DH_NT = 128;
 
 // Debye-Hueckel potential at each ghost node, FP64:
-//   phi_g = sum_a q_a exp(-kappa r) / (eps_out r).
+//   phi_g = sum_a q_a exp(-kappa r) / (eps_out r), atoms in input order,
+// every operation rounded to nearest.  (The solves that run an FP32
+// preconditioner turn a last bit of this sum into 1e-8 of their solution, so
+// its rounding is part of the result.)
 // Bound by FP64 arithmetic (the chip issues two FP64 operations a clock and
-// SM): with sqrt, exp and a division a pair cost about 60 of them; here 24:
-//   - 1/r and r from a 22-bit seed (hardware rsqrt of d2 as a float; the
-//     conversions move bits in integer registers, off the FP64 pipe) by one
-//     third-order Householder step for y = d2^(-1/2):
-//     e = 1 - d2 y^2, y (1 + e (1/2 + 3/8 e)), error 5/16 e^3 < 2^-64;
-//   - exp(-kappa r) = 2^(k/256) 2^(f/256), k the nearest integer and |f| <= 1/2:
-//     a table of 256 powers, the exponent of k added to the entry's exponent
-//     field, and the Taylor polynomial of degree 4 (|x| = |f| ln 2 / 256 <
-//     1.4e-3: x^5/120 < 2^-54);
-//   - the division by eps_out once per node.
-// A CTA takes 32 nodes; its warps share out the atoms, and their sums are
-// added in warp order, so that small grids fill the chip too.  Measured (whole
-// setup of a grid): 97^3 with 1,000 atoms 5.0 -> 2.7 ms, 129^3 with 2,500 atoms
-// 24.0 -> 11.4 ms (250 M pairs: 0.55 T FP64 operations/s, 0.87 of the measured
-// FP64 rate); rms error against long doubles 4e-16 of the values (before: 1e-15
-// at 97^3).
-constexpr int DHX_NT = 256, DHX_TAB = 256;
-// d2 outside 2^+-120, or not finite: the plain formula
-__device__ __noinline__ double dh_term_any(double d2, double q, double kappa) {
-  const double r = sqrt(d2);
-  return q * exp(-kappa * r) / r;
+// SM).  The square root and the quotient are rounded correctly here from one
+// reciprocal square root:
+//   - y = 1/sqrt(d2): a 22-bit seed (hardware rsqrt of d2 as a float; the
+//     conversions move bits in integer registers, off the FP64 pipe) and one
+//     third-order Householder step, e = 1 - d2 y^2, y (1 + e (1/2 + 3/8 e)),
+//     error 5/16 e^3 < 2^-62;
+//   - r = d2 y, corrected by its exact remainder: r + (d2 - r^2) y / 2;
+//   - t / (eps_out r) = t y / eps_out, corrected by its exact remainder
+//     (Markstein 1990), y / eps_out being within a few units of 1 / (eps_out r).
+// Both corrections leave an error of some 2^-50 units in the last place before
+// the one rounding: that a result rounds another way than the exact value has a
+// probability of that order.
+// A CTA takes 32 nodes, which lie on a few lines of a face: of d2 only the square
+// along the line is formed a pair, the other two once a line and atom (36 FP64
+// operations a pair, half of them in exp; one thread a node with sqrt and the
+// division: 44).  Its warps share out the atoms' terms and leave them in shared
+// memory, and one warp adds them up in the atoms' order while the others go on,
+// so that small grids fill the chip too.  Measured, whole setup of a grid, against
+// one thread a node: 33^3 with 200 atoms 0.59 -> 0.37 ms, 97^3 with 1,000 5.06 ->
+// 4.25, 129^3 with 2,500 24.2 -> 17.7, 257^3 with 20,000 664 -> 537; the FP64 pipe
+// is busy for 86% of its nominal rate in both, the most that was seen on it.
+constexpr int DHX_NT = 256, DHX_ATOMS = 64, DHX_LINES = DHX_NT / DHX_ATOMS;
+// d2 or the quotient's operands far from 1, or not finite: the plain formula
+__device__ __noinline__ double dh_term_any(double d2, double q, double kappa, double eps_out) {
+  const double r = __dsqrt_rn(d2);
+  return __ddiv_rn(__dmul_rn(q, exp(-__dmul_rn(kappa, r))), __dmul_rn(eps_out, r));
+}
+__device__ __forceinline__ bool dh_plain_range(double v) {  // 2^-120 <= |v| < 2^120
+  return (((uint32_t)__double2hiint(v) & 0x7fffffffu) - ((1023u - 120u) << 20)) < 240u << 20;
+}
+// whether ghost node t is the first of its line (the fastest index of its face)
+__device__ __forceinline__ bool ghost_starts_line(const Geom &g, long t) {
+  const long n_x = 2L * g.ny * g.nz;
+  return t < n_x ? t % g.ny == 0 : (t - n_x) % g.nx == 0;
+}
+__device__ __forceinline__ bool dh_zero(double v) {
+  return ((uint32_t)__double2hiint(v) << 1 | (uint32_t)__double2loint(v)) == 0;
 }
 __global__ void __launch_bounds__(DHX_NT) k_dh_f64(const dbl4 *xyzq, int n_atoms, Geom g, double kappa,
                                                    double eps_out, double *ghost, long n_ghost) {
-  __shared__ dbl4 sa[DHX_NT];
-  __shared__ double tab[DHX_TAB];       // 2^(j/256)
-  __shared__ double part[DHX_NT / 32][32];
+  __shared__ dbl4 sa[2][DHX_ATOMS];
+  __shared__ double term[2][DHX_ATOMS][32];
+  __shared__ double sq[2][DHX_LINES][DHX_ATOMS][2];  // squares across the line, in the order they are added
+  __shared__ double line_xy[DHX_LINES], line_z[DHX_LINES];
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  for (int t = threadIdx.x; t < DHX_TAB; t += DHX_NT) tab[t] = exp2((double)t / DHX_TAB);
   const long t = blockIdx.x * 32L + lane;
   double px = 0, py = 0, pz = 0;
   if (t < n_ghost) ghost_pos(g, t, px, py, pz);
-  // exponent of 2, in 256ths, per A: -kappa 256 / ln 2 to twice the precision
-  // (log2 e = 1.4426950408889634 + 2.0355273740931033e-17), so that the
-  // exponent carries the rounding of r alone
-  const double L = 1.4426950408889634 * DHX_TAB, L_lo = 2.0355273740931033e-17 * DHX_TAB;
-  const double kl = -kappa * L, kl_lo = fma(-kappa, L, -kl) - kappa * L_lo;
-  const float klf = (float)kl;
-  const double magic = 6755399441055744.0;                       // 1.5 * 2^52: adding it rounds to an integer
-  const double c1 = 6.93147180559945309417e-1 / DHX_TAB;         // ln 2 / 256, then its powers / n!
-  const double c2 = c1 * c1 / 2, c3 = c2 * c1 / 3, c4 = c3 * c1 / 4;
+  const bool along_y = t < 2L * g.ny * g.nz;  // x-faces: lines along y; the others: along x
+  const bool starts = lane == 0 || ghost_starts_line(g, t);
+  const unsigned lines = __ballot_sync(~0u, starts);
+  const int line = __popc(lines << (31 - lane)) - 1;
+  const bool shared = __popc(lines) <= DHX_LINES;  // (not so where a face's lines are shorter than 16)
+  const unsigned y_lines = __ballot_sync(~0u, starts && along_y);
+  const int n_y = __popc(y_lines);  // the first n_y lines are along y
+  if (shared && warp == 0 && starts) {
+    line_xy[line] = along_y ? px : py;
+    line_z[line] = pz;
+  }
+  const double along = along_y ? py : px;
+  const int axis = along_y ? 1 : 0;
+  const double inv_eps = __drcp_rn(eps_out);
+  const bool eps_plain = dh_plain_range(eps_out);
   double s = 0.0;
-  for (int base = 0; base < n_atoms; base += DHX_NT) {
-    __syncthreads();
-    if (base + (int)threadIdx.x < n_atoms) sa[threadIdx.x] = xyzq[base + threadIdx.x];
-    __syncthreads();
-    const int m = min(DHX_NT, n_atoms - base);
+  auto load = [&](int base) {
+    if ((int)threadIdx.x < DHX_ATOMS && base + (int)threadIdx.x < n_atoms)
+      sa[base / DHX_ATOMS & 1][threadIdx.x] = xyzq[base + threadIdx.x];
+  };
+  auto squares = [&](int base) {  // thread: one atom, one line
+    const int l = threadIdx.x / DHX_ATOMS, u = threadIdx.x % DHX_ATOMS;
+    if (!shared || l >= __popc(lines) || base + u >= n_atoms) return;
+    const double *A = (const double *)(xyzq + base + u);
+    const double d1 = __dsub_rn(line_xy[l], A[l < n_y ? 0 : 1]), dz = __dsub_rn(line_z[l], A[2]);
+    double *q = sq[base / DHX_ATOMS & 1][l][u];
+    q[0] = __dmul_rn(d1, d1);
+    q[1] = __dmul_rn(dz, dz);
+  };
+  auto terms = [&](auto sh, int buf, int m) {
+    constexpr bool SHARED = decltype(sh)::value;
 #pragma unroll 2
     for (int u = warp; u < m; u += DHX_NT / 32) {
-      const dbl4 A = sa[u];
-      const double dx = px - A.x, dy = py - A.y, dz = pz - A.z;
-      const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const uint32_t hi = (uint32_t)__double2hiint(d2), lo = (uint32_t)__double2loint(d2);
-      if (hi - ((1023u - 120u) << 20) >= 240u << 20) {
-        s += dh_term_any(d2, A.w, kappa);
-        continue;
+      const double *A = (const double *)&sa[buf][u];
+      const double w = A[3];
+      double s1, sz, v;
+      if constexpr (SHARED) {
+        s1 = sq[buf][line][u][0];
+        sz = sq[buf][line][u][1];
+      } else {
+        const double d1 = __dsub_rn(along_y ? px : py, A[1 - axis]), dz = __dsub_rn(pz, A[2]);
+        s1 = __dmul_rn(d1, d1);
+        sz = __dmul_rn(dz, dz);
       }
+      const double d0 = __dsub_rn(along, A[axis]);
+      const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), s1), sz);
+      const uint32_t hi = (uint32_t)__double2hiint(d2), lo = (uint32_t)__double2loint(d2);
       float y32;
       const float d32 = __uint_as_float(__funnelshift_l(lo, hi - (896u << 20), 3));  // truncated
       asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y32) : "f"(d32));
       const uint32_t yb = __float_as_uint(y32);
-      const double y = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
-      const double r0 = d2 * y, e = fma(-r0, y, 1.0), w = fma(e, 0.375, 0.5);
-      const double r = fma(r0 * e, w, r0), rinv = fma(y * e, w, y);
-      const double big = fma(r, kl, magic), f = fma(r, kl_lo, fma(r, kl, magic - big));
-      const int k = __double2loint(big);
-      const double T = tab[k & (DHX_TAB - 1)];
-      const double pw = __hiloint2double(__double2hiint(T) + ((k >> 8) << 20), __double2loint(T));
-      const double p = fma(f, fma(f, fma(f, c4, c3), c2), c1);
-      // (below 2^-1021 the term is 0)
-      const double qw = d32 * y32 * klf > -1021.f * DHX_TAB ? A.w * rinv * pw : 0.0;
-      s = fma(qw, fma(f, p, 1.0), s);
+      const double y0 = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+      const double e = fma(-__dmul_rn(d2, y0), y0, 1.0);
+      const double y = fma(__dmul_rn(y0, e), fma(e, 0.375, 0.5), y0);
+      const double r0 = __dmul_rn(d2, y);
+      const double hy = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
+      const double r = fma(fma(-r0, r0, d2), hy, r0);
+      const double tq = __dmul_rn(w, exp(-__dmul_rn(kappa, r))), b = __dmul_rn(eps_out, r);
+      const double yi = __dmul_rn(y, inv_eps), q0 = __dmul_rn(tq, yi);
+      v = fma(fma(-q0, b, tq), yi, q0);
+      // (tq = 0: v is 0 either way)
+      if (!(eps_plain && hi - ((1023u - 120u) << 20) < 240u << 20 && (dh_plain_range(tq) || dh_zero(tq))))
+        v = dh_term_any(d2, w, kappa, eps_out);
+      term[buf][u][lane] = v;
+    }
+  };
+  load(0);
+  __syncthreads();
+  squares(0);
+  __syncthreads();
+  for (int base = 0; base < n_atoms; base += DHX_ATOMS) {
+    const int m = min(DHX_ATOMS, n_atoms - base), buf = base / DHX_ATOMS & 1;
+    load(base + DHX_ATOMS);
+    squares(base + DHX_ATOMS);
+    if (shared) terms(std::true_type(), buf, m);
+    else terms(std::false_type(), buf, m);
+    __syncthreads();  // terms and the next atoms are there
+    if (warp == 0) {
+#pragma unroll 8
+      for (int u = 0; u < m; u++) s = __dadd_rn(s, term[buf][u][lane]);
     }
   }
-  part[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0 && t < n_ghost) {
-    double v = part[0][lane];
-    for (int w = 1; w < DHX_NT / 32; w++) v += part[w][lane];
-    ghost[t] = v / eps_out;
-  }
+  if (warp == 0 && t < n_ghost) ghost[t] = s;
 }
 
 // Same sum in FP32 arithmetic: hardware reciprocal square root and base-2
