@@ -793,7 +793,7 @@ static bool use_resident(pb_grid *g, const pb_solve_opts *o, int mode, int coef)
     g->res_mode = mode;
     g->res_coef = coef;
     g->res_fits = resident_plan(g->d.nx, g->d.ny, g->d.nz, mode, coef, g->ctx->num_sms,
-                                g->ctx->max_smem - RES_STATIC_SMEM, &g->res_plan);
+                                g->ctx->max_smem, &g->res_plan);
   }
   return g->res_fits;
 }

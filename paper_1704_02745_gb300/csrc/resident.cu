@@ -1,6 +1,6 @@
 // resident.cu -- one inner CG solve (Sec. 2.2 preconditioned CG, Sec. 2.4
-// Jacobi, operator of Eq. 3-4) of a single grid in one cooperative kernel that
-// keeps the vectors on the chip.
+// Jacobi, operator of Eq. 3-4) of a grid in one cooperative kernel that keeps
+// the vectors on the chip; and of several grids of a batch side by side.
 //
 // What bounds the two-pass form (solve.cu) on one grid is not its bytes: a
 // 129^3 iteration moves 82 MB, 12 us at the measured copy rate, and takes 40
@@ -19,8 +19,8 @@
 //     neighbours' boundary z and keeps its own copy of their p), Ap and p.Ap;
 //     a grid-wide sum; r = M z - alpha Ap, z = M^-1 r, r.z, r.r, the
 //     boundary z written out; a grid-wide sum.  The same operations per node
-//     in the same order as cg_tile; only the partial sums are grouped by
-//     brick.
+//     as cg_tile, up to the order in which a surface node's six edges are
+//     added; the partial sums are grouped by brick.
 //   - the grid-wide sum is the barrier: each CTA stores its sum and an epoch as
 //     one 16-byte word in a line of its own, and every CTA polls all CTAs'
 //     words, one thread each, and adds them in CTA order, so every CTA holds
@@ -36,6 +36,8 @@
 
 #include <algorithm>
 #include <climits>
+#include <iterator>
+#include <type_traits>
 
 #include "coef.cuh"
 #include "pb_internal.cuh"
@@ -241,9 +243,9 @@ __device__ __forceinline__ bool await_word(const Packet *words, int c, Sum<T> (&
 // At least four warps a CTA.  Out of line: the kernel's code is larger than the
 // instruction caches that feed it.
 template <typename T, int N, int NTH>
-__device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, uint32_t epoch, bool publish, int *err,
-                                      SumScratch<T, NTH> &S, bool first) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, ncta = gridDim.x;
+__device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, int cta, int ncta, uint32_t epoch, bool publish,
+                                         int *err, SumScratch<T, NTH> &S, bool first) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   S.part[0][threadIdx.x] = v0;
   if (N == 2) S.part[1][threadIdx.x] = v1;
   __syncthreads();
@@ -269,7 +271,7 @@ __device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, uint32_t epo
       Sum<T> s[N];
 #pragma unroll
       for (int n = 0; n < N; n++) s[n] = S.block[n];
-      wire_store(words + (size_t)PACKET_STRIDE * blockIdx.x, s, epoch);
+      wire_store(words + (size_t)PACKET_STRIDE * cta, s, epoch);
     }
   }
   const int pollers = min(nw - 1, (ncta + 31) >> 5);  // warps that poll
@@ -505,9 +507,19 @@ __device__ __forceinline__ Q4<T> packed_ap(bool simple, bool carried, uint32_t c
 // solves (KEEP), whose arithmetic is what they wait for, and formed again from
 // p by FP32 solves (8 B a node of L2 traffic less).  PER: periodic axes.
 constexpr int RES_YH = 3;  // y-halo groups a thread can own
+// CTAs on an SM: the small builds, of batches, come in pairs, one computing while
+// the other waits for its sums
+constexpr int ctas_per_sm(int threads) { return threads <= 256 ? 2 : 1; }
 
-template <typename T, int CM, int G, int NTH, bool PER>
-__global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ ResArgs R) {
+template <typename T, int CM, int G, int NTH, bool PER, typename W>
+__global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __grid_constant__ W wave) {
+  int n_grid = 0, cta = blockIdx.x, ncta = gridDim.x;  // this CTA's grid, its number there
+  if constexpr (std::is_same_v<W, ResWave>) {
+    while (cta >= wave.first[n_grid + 1]) n_grid++;
+    ncta = wave.first[n_grid + 1] - wave.first[n_grid];
+    cta -= wave.first[n_grid];
+  }
+  const ResArgs &R = wave.grid[n_grid];
   constexpr bool SEP = sizeof(T) == 4;  // FP32 inner solves accumulate into d
   constexpr bool REG = G > 0, KEEP = REG || sizeof(T) == 8;
   // planes whose loads are issued together
@@ -521,7 +533,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
   if (*(volatile int *)&Sp->phase != PH_START) return;  // nothing to solve (the same for every CTA)
   if (threadIdx.x == 0) S.failed = 0;
   const int by = R.by, gpr = R.gpr, rp = 4 * gpr + 4, ps_plane = (by + 2) * rp;
-  const int cy = blockIdx.x % R.nby, cz = blockIdx.x / R.nby;
+  const int cy = cta % R.nby, cz = cta / R.nby;
   const int y0 = cy * by, z0 = cz * R.bz;
   const int ny = R.ny, nz = R.nz, nx = R.nx, px = R.px;
   const int rows = min(by, ny - y0), kn = min(R.bz, nz - z0);
@@ -582,7 +594,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
   const uint32_t own_lanes = __ballot_sync(0xffffffffu, own);
   const bool left_edge = xg == 0 || (threadIdx.x & 31) == 0, right_edge = xg == gpr - 1 || (threadIdx.x & 31) == 31;
   if (threadIdx.x == 0) {
-    const int b = blockIdx.x, nby = R.nby, nbz = R.nbz;
+    const int b = cta, nby = R.nby, nbz = R.nbz;
     S.neighbour[0] = cy > 0 ? b - 1 : PER ? b + nby - 1 : -1;
     S.neighbour[1] = cy < nby - 1 ? b + 1 : PER ? b - nby + 1 : -1;
     S.neighbour[2] = cz > 0 ? b - nby : PER ? b + (nbz - 1) * nby : -1;
@@ -627,7 +639,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
   int iter = 0, total = Sp->total_iter, status = Sp->status, phase = PH_INNER;
   const int max_iter = I.max_iter;
   Packet *const words_a = (Packet *)R.packets;  // p.Ap
-  Packet *const words_b = words_a + (size_t)PACKET_STRIDE * gridDim.x;  // r.z, r.r
+  Packet *const words_b = words_a + (size_t)PACKET_STRIDE * ncta;  // r.z, r.r
   auto code_of = [&](int k) -> uint32_t {
     if (CM != COEF_PACKED) return 0u;
     return REG ? cs[k * blockDim.x] : __ldg((const uint32_t *)(R.code + e0 + k * plane));
@@ -806,7 +818,8 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
     }
     // (the first sum also orders reading the residual pass's z before a
     // neighbour's G = 0 build overwrites it)
-    if (!grid_sum<T, 1, NTH>(total_of(acc) * scale_t, (T)0, words_a, 2u * iter + 1u, iter == 0, R.err, S, iter == 0))
+    if (!grid_sum<T, 1, NTH>(total_of(acc) * scale_t, (T)0, words_a, cta, ncta, 2u * iter + 1u, iter == 0, R.err, S,
+                             iter == 0))
       return;
     if (!(lead(S.grid[0]) > (T)0) || !isfinite(lead(S.alpha))) {
       status = 6;  // PB_ERR_BREAKDOWN
@@ -860,8 +873,8 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
         }
       }
     }
-    if (!grid_sum<T, 2, NTH>(total_of(rz) * scale_t, total_of(rr) * scale_t, words_b, 2u * iter + 2u, true, R.err, S,
-                             false))
+    if (!grid_sum<T, 2, NTH>(total_of(rz) * scale_t, total_of(rr) * scale_t, words_b, cta, ncta, 2u * iter + 2u, true,
+                             R.err, S, false))
       return;
     if (!isfinite(lead(S.grid[0])) || !isfinite(lead(S.grid[1]))) {
       status = 6;
@@ -892,7 +905,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
         if (k < kn) q_store(gd + e0 + k * plane, d[k]);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (cta == 0 && threadIdx.x == 0) {
     if (phase == PH_RESID) {
       Sp->alpha = value(S.alpha);
       Sp->beta = value(S.beta);
@@ -904,7 +917,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_resident(const __grid_constant__ 
     Sp->total_iter = total;
     Sp->status = status;
     Sp->phase = phase;
-    if (phase == PH_RESID) R.resid_list[atomicAdd(R.resid_pending, 1)] = 0;
+    if (phase == PH_RESID) R.resid_list[atomicAdd(R.resid_pending, 1)] = R.slot;
   }
 }
 
@@ -919,14 +932,20 @@ struct Build {
 // Builds by planes a thread owns (0: any); threads: the most whose registers fit one SM.
 constexpr Build F32_BUILDS[] = {{2, 512}, {4, 512}, {5, 512}, {6, 512}, {8, 512}, {12, 384}, {0, 1024}};
 constexpr Build F64_BUILDS[] = {{0, 512}};
+// Of a batch: an iteration of two grids of 97^3 takes 10.8 us in the pairs of {8, 256},
+// 12.1 in {8, 512}, one of them alone 9.1 and 9.
+constexpr Build BATCH_BUILDS[] = {{8, 512}, {12, 384}, {8, 256}, {12, 192}};  // FP32 grids of a batch, packed codes
 
 size_t p_bytes(int by, int bz, int gpr, int es) {
   return ((size_t)((size_t)(bz + 2) * (by + 2) * (4 * gpr + 4) + 4) * es + 15) / 16 * 16;
 }
 
-template <typename T, int CM, int G, int NTH>
-cudaError_t launch_build(const ResPlan &P, const ResArgs &R, bool per, cudaStream_t st) {
-  auto *k = per ? k_cg_resident<T, CM, G, NTH, true> : k_cg_resident<T, CM, G, NTH, false>;
+struct Shape {  // of a launch
+  int ctas, threads;
+  size_t smem;
+};
+template <typename W, typename K>
+cudaError_t launch_kernel(K *k, const Shape &P, const W &wave, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -939,12 +958,25 @@ cudaError_t launch_build(const ResPlan &P, const ResArgs &R, bool per, cudaStrea
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, R);
+  return cudaLaunchKernelEx(&cfg, k, wave);
+}
+// Shared memory: p, then (G > 0) Ap, then (packed codes) the code words, a
+// thread's groups each.
+size_t off_codes(const ResPlan &P, int es, int threads) {
+  return (size_t)P.off_ap + (P.planes ? (size_t)4 * es * P.bz * threads : 0);
+}
+size_t smem_of(const ResPlan &P, int es, int coef, int threads) {
+  return off_codes(P, es, threads) + (P.planes && coef == COEF_PACKED ? (size_t)4 * P.bz * threads : 0);
+}
+template <typename T, int CM, int G, int NTH, typename W = ResOne>
+cudaError_t launch_build(const Shape &P, const W &wave, bool per, cudaStream_t st) {
+  return per ? launch_kernel<W>(k_cg_resident<T, CM, G, NTH, true, W>, P, wave, st)
+             : launch_kernel<W>(k_cg_resident<T, CM, G, NTH, false, W>, P, wave, st);
 }
 
 template <int CM>
-cudaError_t launch_f32(const ResPlan &P, const ResArgs &R, bool per, cudaStream_t st) {
-  switch (P.build) {
+cudaError_t launch_f32(int build, const Shape &P, const ResOne &R, bool per, cudaStream_t st) {
+  switch (build) {
     case 0: return launch_build<float, CM, 2, 512>(P, R, per, st);
     case 1: return launch_build<float, CM, 4, 512>(P, R, per, st);
     case 2: return launch_build<float, CM, 5, 512>(P, R, per, st);
@@ -955,69 +987,23 @@ cudaError_t launch_f32(const ResPlan &P, const ResArgs &R, bool per, cudaStream_
   }
 }
 template <int CM>
-cudaError_t launch_f64(const ResPlan &P, const ResArgs &R, bool per, cudaStream_t st) {
+cudaError_t launch_f64(const Shape &P, const ResOne &R, bool per, cudaStream_t st) {
   return launch_build<double, CM, 0, 512>(P, R, per, st);
 }
 
-}  // namespace
-
-bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, ResPlan *out) {
-  const int es = mode == MODE_F64 ? 8 : 4, gpr = (nx + 3) / 4;
-  const Build *builds = mode == MODE_F64 ? F64_BUILDS : F32_BUILDS;
-  const int nb = mode == MODE_F64 ? (int)(sizeof(F64_BUILDS) / sizeof(Build)) : (int)(sizeof(F32_BUILDS) / sizeof(Build));
-  bool found = false;
-  double best = 0;
-  for (int b = 0; b < nb; b++) {
-    const Build &B = builds[b];
-    for (int bym = 1; bym * gpr <= B.threads && bym <= ny; bym++) {
-      for (int bzm = 1; bzm <= (B.G ? B.G : nz) && bzm <= nz; bzm++) {
-        const int nby = (ny + bym - 1) / bym, nbz = (nz + bzm - 1) / bzm;
-        if ((long)nby * nbz > std::min(num_sms, RES_MAX_CTAS)) continue;
-        const int by = (ny + nby - 1) / nby, bz = (nz + nbz - 1) / nbz;
-        const int threads = std::max(128, (by * gpr + 31) / 32 * 32);  // four warps: grid_sum
-        if (threads > B.threads || bz > 32 || 2 * bz * gpr > RES_YH * threads) continue;
-        const size_t off_ap = p_bytes(by, bz, gpr, es), cb = (size_t)4 * bz * threads;
-        const size_t pb = off_ap + (B.G ? (size_t)4 * es * bz * threads : 0);
-        const size_t smem = pb + (B.G && coef == COEF_PACKED ? cb : 0);
-        if (smem > (size_t)max_smem) continue;
-        // Cycles of an iteration: a plane costs its groups' issue slots on four
-        // schedulers and a latency, more in the builds whose registers spill;
-        // the two grid-wide sums.  (Measured best and the model's choice differ
-        // by 3% at most on cubes of 33 to 145 nodes a side.)
-        const double group = es == 8 ? 900.0 : coef == COEF_PACKED ? 150.0 : 200.0;
-        const double spill = B.G == 0 ? 2.5 : B.G >= 8 ? 1.2 : B.G >= 5 && coef != COEF_PACKED ? 1.15 : 1.0;
-        const double warps = threads / 32.0;
-        const double cost = spill * bz * (warps / 4.0 * group + 400.0) + 6000.0 + 6.0 * nby * nbz;
-        if (found && cost >= best) continue;
-        found = true;
-        best = cost;
-        out->build = b;
-        out->by = by;
-        out->bz = bz;
-        out->nby = (ny + by - 1) / by;
-        out->nbz = (nz + bz - 1) / bz;
-        out->ctas = out->nby * out->nbz;
-        out->threads = threads;
-        out->gpr = gpr;
-        out->off_ap = (int)off_ap;
-        out->off_codes = (int)pb;
-        out->smem = smem;
-      }
-    }
+cudaError_t launch_batch(int build, const Shape &P, const ResWave &R, bool per, cudaStream_t st) {
+  switch (build) {
+    case 0: return launch_build<float, COEF_PACKED, 8, 512>(P, R, per, st);
+    case 1: return launch_build<float, COEF_PACKED, 12, 384>(P, R, per, st);
+    case 2: return launch_build<float, COEF_PACKED, 8, 256>(P, R, per, st);
+    default: return launch_build<float, COEF_PACKED, 12, 192>(P, R, per, st);
   }
-  return found;
 }
 
-size_t resident_packet_bytes(int num_sms) { return 2 * PACKET_STRIDE * sizeof(Packet) * (size_t)num_sms; }
-
-cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, void *packets, size_t packet_bytes,
-                            cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(packets, 0, packet_bytes, st);  // epochs count from 1 in every launch
-  if (e != cudaSuccess) return e;
-  const int mode = I.mode, coef = I.coef;
-  const bool periodic = I.periodic != 0;
+// Kernel arguments of one grid; threads: of the launch.
+ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &B, void *packets, int slot, int threads) {
   ResArgs R;
-  R.inst = B.inst;
+  R.inst = dI;
   R.packets = packets;
   R.err = B.error;
   R.resid_pending = B.resid_pending;
@@ -1042,15 +1028,108 @@ cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, voi
   R.gpr = P.gpr;
   // g / gpr = umulhi(g, magic) for g * gpr < 2^32
   R.gpr_magic = P.gpr > 1 ? (uint32_t)(((1ull << 32) + P.gpr - 1) / P.gpr) : 0u;
-  R.off_codes = P.off_codes;
   R.off_ap = P.off_ap;
-  if (mode == MODE_F64) {
-    if (coef == COEF_F64) return launch_f64<COEF_F64>(P, R, periodic, st);
-    return launch_f64<COEF_PACKED>(P, R, periodic, st);
+  R.off_codes = off_codes(P, I.mode == MODE_F64 ? 8 : 4, threads);
+  R.slot = slot;
+  return R;
+}
+
+}  // namespace
+
+// The plan of least cost: of an iteration (alone), or of an iteration of as many
+// such grids as the device holds at once, a grid.
+static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, bool alone, ResPlan *out) {
+  const int es = mode == MODE_F64 ? 8 : 4, gpr = (nx + 3) / 4;
+  const Build *builds = !alone ? BATCH_BUILDS : mode == MODE_F64 ? F64_BUILDS : F32_BUILDS;
+  const int nb = !alone ? std::size(BATCH_BUILDS) : mode == MODE_F64 ? std::size(F64_BUILDS) : std::size(F32_BUILDS);
+  bool found = false;
+  double best = 0;
+  for (int b = 0; b < nb; b++) {
+    const Build &B = builds[b];
+    const int per_sm = ctas_per_sm(B.threads), room = per_sm * num_sms;
+    // (an SM keeps 1 KB of each CTA's shared memory to itself)
+    const int smem = (max_smem + 1024) / per_sm - 1024 - RES_STATIC_SMEM / per_sm;
+    for (int bym = 1; bym * gpr <= B.threads && bym <= ny; bym++) {
+      for (int bzm = 1; bzm <= (B.G ? B.G : nz) && bzm <= nz; bzm++) {
+        const int nby = (ny + bym - 1) / bym, nbz = (nz + bzm - 1) / bzm;
+        if ((long)nby * nbz > std::min(room, RES_MAX_CTAS)) continue;
+        ResPlan P;
+        P.build = b;
+        P.planes = B.G;
+        P.by = (ny + nby - 1) / nby;
+        P.bz = (nz + nbz - 1) / nbz;
+        P.gpr = gpr;
+        P.threads = std::max(128, (P.by * gpr + 31) / 32 * 32);  // four warps: grid_sum
+        if (P.threads > B.threads || P.bz > 32 || 2 * P.bz * gpr > RES_YH * P.threads) continue;
+        P.off_ap = (int)p_bytes(P.by, P.bz, gpr, es);
+        // (in a batch the launch has the threads of its largest plan)
+        if ((long)smem_of(P, es, coef, alone ? P.threads : B.threads) > smem) continue;
+        P.nby = (ny + P.by - 1) / P.by;
+        P.nbz = (nz + P.bz - 1) / P.bz;
+        P.ctas = P.nby * P.nbz;
+        P.room = room;
+        // Cycles of an iteration: a plane costs its groups' issue slots on four
+        // schedulers and a latency, more in the builds whose registers spill;
+        // the two grid-wide sums.  (Measured best and the model's choice differ
+        // by 3% at most on cubes of 33 to 145 nodes a side.)
+        const double group = es == 8 ? 900.0 : coef == COEF_PACKED ? 150.0 : 200.0;
+        const double spill = B.G == 0 ? 2.5 : B.G >= 8 ? 1.2 : B.G >= 5 && coef != COEF_PACKED ? 1.15 : 1.0;
+        const double issue = spill * P.bz * P.threads / 32.0 / 4.0 * group;
+        double cost = issue + spill * P.bz * 400.0 + 6000.0 + 6.0 * nby * nbz;
+        if (!alone) cost = std::max(cost, per_sm * issue + 2000.0) / (room / P.ctas);
+        if (found && cost >= best) continue;
+        found = true;
+        best = cost;
+        *out = P;
+      }
+    }
   }
-  if (coef == COEF_F32) return launch_f32<COEF_F32>(P, R, periodic, st);
-  if (coef == COEF_BF16) return launch_f32<COEF_BF16>(P, R, periodic, st);
-  return launch_f32<COEF_PACKED>(P, R, periodic, st);
+  return found;
+}
+bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, ResPlan *out) {
+  return best_plan(nx, ny, nz, mode, coef, num_sms, max_smem, true, out);
+}
+bool resident_batch_plan(int nx, int ny, int nz, int num_sms, int max_smem, ResPlan *out) {
+  return best_plan(nx, ny, nz, MODE_F32_REFINE, COEF_PACKED, num_sms, max_smem, false, out);
+}
+
+size_t resident_packet_bytes(int ctas) { return 2 * PACKET_STRIDE * sizeof(Packet) * (size_t)ctas; }
+
+cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, void *packets, size_t packet_bytes,
+                            cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(packets, 0, packet_bytes, st);  // epochs count from 1 in every launch
+  if (e != cudaSuccess) return e;
+  const bool per = I.periodic != 0;
+  ResOne R;
+  R.grid[0] = grid_args(P, I, B.inst, B, packets, 0, P.threads);
+  const Shape L{P.ctas, P.threads, smem_of(P, I.mode == MODE_F64 ? 8 : 4, I.coef, P.threads)};
+  if (I.mode == MODE_F64) {
+    if (I.coef == COEF_F64) return launch_f64<COEF_F64>(L, R, per, st);
+    return launch_f64<COEF_PACKED>(L, R, per, st);
+  }
+  if (I.coef == COEF_F32) return launch_f32<COEF_F32>(P.build, L, R, per, st);
+  if (I.coef == COEF_BF16) return launch_f32<COEF_BF16>(P.build, L, R, per, st);
+  return launch_f32<COEF_PACKED>(P.build, L, R, per, st);
+}
+
+cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *const *I, const int *slot,
+                                  const Batch &B, void *packets, size_t packet_bytes, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(packets, 0, packet_bytes, st);
+  if (e != cudaSuccess) return e;
+  Shape L{0, 0, 0};
+  for (int k = 0; k < n; k++) L.threads = std::max(L.threads, P[k]->threads);
+  ResWave W;
+  W.n = n;
+  for (int k = 0; k < n; k++) {
+    W.first[k] = L.ctas;
+    W.grid[k] = grid_args(*P[k], *I[k], B.inst + slot[k], B, (Packet *)packets + (size_t)2 * PACKET_STRIDE * L.ctas,
+                          slot[k], L.threads);
+    L.ctas += P[k]->ctas;
+    L.smem = std::max(L.smem, smem_of(*P[k], 4, COEF_PACKED, L.threads));
+  }
+  for (int k = n; k <= RES_MAX_GRIDS; k++) W.first[k] = L.ctas;
+  const bool per = I[0]->periodic != 0;
+  return launch_batch(P[0]->build, L, W, per, st);
 }
 
 }  // namespace pb

@@ -8,9 +8,10 @@ struct ResPlan {  // how a grid is cut into bricks, one CTA each
   int build = 0;              // index of the kernel build
   int by = 0, bz = 0;         // rows and planes of a brick
   int nby = 0, nbz = 0, ctas = 0;
+  int room = 0;               // CTAs of its build that the device holds at once
   int threads = 0, gpr = 0;   // groups of four x nodes per row
-  int off_codes = 0, off_ap = 0;
-  size_t smem = 0;
+  int planes = 0;             // planes a thread can own (0: any number)
+  int off_ap = 0;             // offset of Ap in shared memory (p before it)
 };
 struct ResArgs {  // kernel arguments
   const Inst *inst;
@@ -23,14 +24,35 @@ struct ResArgs {  // kernel arguments
   int nx, ny, nz, px;
   uint32_t gpr_magic;  // for division by gpr
   int by, bz, nby, nbz, gpr, off_codes, off_ap;
+  int slot;            // its place among the batch's instances
+};
+// The grids of a launch, a run of CTAs each: grid n has CTAs first[n] .. first[n + 1] - 1.
+constexpr int RES_MAX_GRIDS = 16;
+struct ResWave {
+  int n;
+  int first[RES_MAX_GRIDS + 1];
+  ResArgs grid[RES_MAX_GRIDS];
+};
+struct ResOne {  // a launch over one grid
+  ResArgs grid[1];
 };
 
-constexpr int RES_STATIC_SMEM = 16384;  // more than the kernel's static shared memory
+constexpr int RES_STATIC_SMEM = 16384;  // more than the kernel's static shared memory (half: of the builds in pairs)
+constexpr int RES_MAX_PER_SM = 2;       // CTAs of a build on an SM at most
 
-// Plan of a grid for num_sms SMs of max_smem bytes a CTA; false: the grid does
+// Plan of a grid for num_sms SMs of max_smem bytes a CTA (the largest one CTA
+// may ask for); false: the grid does
 // not fit (the two-pass form runs).
 bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, ResPlan *out);
-size_t resident_packet_bytes(int num_sms);
+size_t resident_packet_bytes(int ctas);  // of a launch
+// Plan of a grid of a batch: for the most such grids at once (it does not depend
+// on what else runs, and so neither do the grid's sums).  FP32 with packed codes only.
+bool resident_batch_plan(int nx, int ny, int nz, int num_sms, int max_smem, ResPlan *out);
+// Inner solves of n <= RES_MAX_GRIDS instances of a batch (slot[k], descriptor
+// *I[k] on the host, plans of one build, all periodic or none) that are in
+// their start phase, side by side: at most the plans' room CTAs together.
+cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *const *I, const int *slot,
+                                  const Batch &B, void *packets, size_t packet_bytes, cudaStream_t st);
 // One inner solve of the batch's only instance (I: its descriptor on the host)
 // if it is in its start phase.
 cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, void *packets, size_t packet_bytes,

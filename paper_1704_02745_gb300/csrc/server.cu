@@ -15,9 +15,10 @@
 //      stencil tiles of every active grid, largest first, each grid's partial
 //      sums at its own offset, so its reductions are summed in a fixed order
 //      whatever else runs;
-//   4. queues a captured device graph of `ticks` phase ticks over the whole
-//      batch (finished grids are skipped by their convergence mask) and a copy
-//      of all grids' scalars;
+//   4. queues whole inner solves of the batch's grids, kept on the chip
+//      (run_resident_round), or else a captured device graph of `ticks` phase
+//      ticks over the whole batch (finished grids are skipped by their
+//      convergence mask), and a copy of all grids' scalars;
 //   5. while that graph runs, reads the scalars the previous round's graph
 //      left, queues the energy (and phi) of the solves that finished in it on
 //      the copy stream, beside the running graph, and hands out the results
@@ -40,6 +41,7 @@
 #include "pb.h"
 #include "pb_host.h"
 #include "pb_internal.cuh"
+#include "resident.cuh"
 #include "solve.cuh"
 
 using namespace pb;
@@ -141,6 +143,10 @@ struct Slot {
   Request req;
   bool warm = false;
   uint64_t first_round = 0;   // round whose graph first runs the current solve
+  Inst inst;                  // its descriptor, as last uploaded
+  ResPlan res_plan;           // plan of its resident inner solves
+  bool res_fits = false;
+  bool ticked = false;        // phase ticks have run on the current solve: it may be inside an inner solve
 };
 
 // A finished solve whose energy (and phi) are queued behind the running graph.
@@ -199,6 +205,8 @@ struct pb_server {
   Inst *d_inst = nullptr;
   int *d_counts = nullptr, *d_list = nullptr, *d_err = nullptr;
   int *d_rlist = nullptr;  // instances waiting for a residual pass
+  void *d_packets = nullptr;   // words of the resident inner solves (resident.cu)
+  bool resident_off = false;   // the device refused a cooperative launch
   Item *d_st = nullptr;
   double *d_st_part = nullptr, *d_rs_part = nullptr;
   size_t cap_st = 0, cap_rs = 0;
@@ -375,6 +383,9 @@ std::vector<int> admit(pb_server *s) {
       cudaEventRecord(s->ev_idle[j], s->stream);  // its workspace clears
       cudaEventRecord(s->ev_energy[j], s->stream);
       Slot &sl = s->slots[j];
+      sl.res_fits = s->mode != MODE_F64 && s->coef == COEF_PACKED &&
+                    resident_batch_plan(g->d.nx, g->d.ny, g->d.nz, s->ctx->num_sms, s->ctx->max_smem,
+                                        &sl.res_plan);
       sl.g = g;
       sl.traj = rq.traj;
       sl.bytes = rq.bytes;
@@ -483,6 +494,7 @@ bool rebuild_batch(pb_server *s, Stage &sg, bool *graph_stale) {
     if (pb_make_inst(g, &s->opts, s->mode, s->coef, I)) return false;
     I.s = s->d_scal + j;
     I.ap = nullptr;  // the update pass forms Ap again from p (k_update_tile)
+    s->slots[j].inst = I;
     I.st_base = st_off;
     I.rs_base = rs_off;
     rs_off += g->n_rs;
@@ -554,24 +566,96 @@ bool rebuild_batch(pb_server *s, Stage &sg, bool *graph_stale) {
   return true;
 }
 
+Batch server_batch(const pb_server *s) {
+  Batch B;
+  B.inst = s->d_inst;
+  B.st_items = s->d_st;
+  B.ch_items = nullptr;
+  B.n_items = s->d_counts;
+  B.work = (unsigned *)(s->d_counts + 4);
+  B.resid_pending = s->d_counts + 2;
+  B.resid_list = s->d_rlist;
+  B.rs_part = s->d_rs_part;
+  B.st_part = s->d_st_part;
+  B.ch_part = nullptr;
+  B.error = s->d_err;
+  return B;
+}
+
+// A round of whole inner solves instead of ticks: every grid of the batch has
+// a plan that keeps it on the chip, and none is inside an inner solve of ticks.
+// The grids run side by side, several to a cooperative launch, each on the SMs
+// its plan asks for; finished ones take none (the host reads the last round's
+// phases first, some tens of us in rounds of milliseconds).  Ticks are bound by
+// their bytes while many grids run and by latency when few are left; this form
+// by a CTA's chain of latencies, of which two CTAs an SM hide half.  Measured,
+// bursts to 1e-9, ticks -> here: one grid of 97^3 32.4 -> 3.9 ms; 32 of 49^3
+// 35.3 -> 10.6, of 97^3 98.8 -> 70.3, of 113^3 143 -> 139, of 129^3 204 -> 167;
+// 256 of 65^3 200 -> 133; 32 with wrap of 97x81x113 284 -> 93.  A batch with a
+// grid that does not fit (some 2.5 M nodes) runs in ticks: as many bytes a
+// second as this form needs for its share, and no grid waits for another.
+bool can_run_resident(const pb_server *s, const std::vector<int> &active) {
+  if (s->resident_off || s->mode == MODE_F64) return false;
+  for (int j : active)
+    if (!s->slots[j].res_fits || s->slots[j].ticked) return false;
+  return true;
+}
+
+// The residual pass, an inner solve of each grid of `run`, the residual pass.
+// ticks: nothing ran (the device refused the launch), ticks have to.
+bool run_resident_round(pb_server *s, std::vector<int> run, bool *ticks) {
+  *ticks = false;
+  const Batch B = server_batch(s);
+  const size_t bytes = resident_packet_bytes(RES_MAX_PER_SM * s->ctx->num_sms);
+  if (!s->d_packets && pb_dalloc(&s->d_packets, bytes)) {
+    s->resident_off = *ticks = true;
+    return true;
+  }
+  if (!cuda_ok(launch_phase(B, s->mode, s->coef, s->kg, 4, s->stream), s, "residual pass")) return false;
+  // launches: grids of one build, largest first, each into the first with room
+  struct Launch {
+    int ctas = 0;
+    std::vector<int> slots;
+  };
+  auto kind = [&](int j) { return 2 * s->slots[j].res_plan.build + (s->slots[j].g->d.periodic ? 1 : 0); };
+  std::stable_sort(run.begin(), run.end(), [&](int a, int b) {
+    return kind(a) != kind(b) ? kind(a) < kind(b) : s->slots[a].res_plan.ctas > s->slots[b].res_plan.ctas;
+  });
+  std::vector<Launch> launches;
+  for (int j : run) {
+    const int ctas = s->slots[j].res_plan.ctas;
+    auto it = std::find_if(launches.begin(), launches.end(), [&](const Launch &l) {
+      return kind(l.slots[0]) == kind(j) && l.ctas + ctas <= s->slots[j].res_plan.room && (int)l.slots.size() < RES_MAX_GRIDS;
+    });
+    if (it == launches.end()) it = launches.insert(launches.end(), Launch());
+    it->ctas += ctas;
+    it->slots.push_back(j);
+  }
+  for (const Launch &l : launches) {
+    const ResPlan *P[RES_MAX_GRIDS];
+    const Inst *I[RES_MAX_GRIDS];
+    const int n = (int)l.slots.size();
+    for (int k = 0; k < n; k++) {
+      P[k] = &s->slots[l.slots[k]].res_plan;
+      I[k] = &s->slots[l.slots[k]].inst;
+    }
+    if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, s->stream) != cudaSuccess) {
+      cudaGetLastError();  // ticks go on from the state the residual pass left
+      s->resident_off = *ticks = true;
+      return true;
+    }
+  }
+  s->ctx->stats->launches += 2 + launches.size();
+  return cuda_ok(launch_phase(B, s->mode, s->coef, s->kg, 4, s->stream), s, "residual pass");
+}
+
 bool run_graph(pb_server *s, bool stale) {
   if (stale && s->graph) {
     cudaGraphExecDestroy(s->graph);
     s->graph = nullptr;
   }
   if (!s->graph) {
-    Batch B;
-    B.inst = s->d_inst;
-    B.st_items = s->d_st;
-    B.ch_items = nullptr;
-    B.n_items = s->d_counts;
-    B.work = (unsigned *)(s->d_counts + 4);
-    B.resid_pending = s->d_counts + 2;
-    B.resid_list = s->d_rlist;
-    B.rs_part = s->d_rs_part;
-    B.st_part = s->d_st_part;
-    B.ch_part = nullptr;
-    B.error = s->d_err;
+    const Batch B = server_batch(s);
     cudaGraph_t g;
     if (!cuda_ok(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal), s, "capture"))
       return false;
@@ -740,18 +824,7 @@ double launch_bytes(pb_server *s, const std::vector<int> &active, int which) {
 // before each launch.
 bool run_profiled(pb_server *s, const std::vector<int> &active, pb_kernel_profile &prof,
                   int ticks) {
-  Batch B;
-  B.inst = s->d_inst;
-  B.st_items = s->d_st;
-  B.ch_items = nullptr;
-  B.n_items = s->d_counts;
-  B.work = (unsigned *)(s->d_counts + 4);
-  B.resid_pending = s->d_counts + 2;
-  B.resid_list = s->d_rlist;
-  B.rs_part = s->d_rs_part;
-  B.st_part = s->d_st_part;
-  B.ch_part = nullptr;
-  B.error = s->d_err;
+  const Batch B = server_batch(s);
   const int hi = *std::max_element(active.begin(), active.end()) + 1;
   for (int t = 0; t < 3 * ticks; t++) {
     const int which = t % 3 == 0 ? 4 : t % 3 == 1 ? 1 : 2;
@@ -888,6 +961,7 @@ void worker_main(pb_server *s) {
       }
       if (q != cudaSuccess) cuda_ok(q, s, "setup");
       s->slots[j].pending = false;
+      s->slots[j].ticked = false;
       s->slots[j].first_round = s->round;
       started.push_back(j);
       pending.erase(pending.begin() + k);
@@ -974,16 +1048,29 @@ void worker_main(pb_server *s) {
       if (!active.empty() && !rebuild_batch(s, sg, &graph_stale)) break;
     }
     if (want_tune) {
+      for (int j : active) s->slots[j].ticked = true;
       if (!tune_batch(s, sg, active, &graph_stale)) break;
       if (!rebuild_batch(s, sg, &graph_stale)) break;
     }
     bool ran = false;
     if (!active.empty()) {
-      if (s->profiling.load()) {
-        if (!run_profiled(s, active, s->prof, s->ticks)) break;
-      } else {
-        if (!run_graph(s, graph_stale)) break;
-        graph_stale = false;
+      bool ticks = s->profiling.load() || !can_run_resident(s, active);
+      if (!ticks) {
+        // what the last round left: grids that finished in it take no SMs
+        if (prev_graph && !cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) break;
+        std::vector<int> run;
+        for (int j : active)
+          if (s->slots[j].first_round == s->round || !prev_graph || sp.scal[j].phase != PH_DONE) run.push_back(j);
+        if (!run_resident_round(s, run, &ticks)) break;
+      }
+      if (ticks) {
+        for (int j : active) s->slots[j].ticked = true;
+        if (s->profiling.load()) {
+          if (!run_profiled(s, active, s->prof, s->ticks)) break;
+        } else {
+          if (!run_graph(s, graph_stale)) break;
+          graph_stale = false;
+        }
       }
       const int hi = *std::max_element(active.begin(), active.end()) + 1;
       cudaMemcpyAsync(sg.scal, s->d_scal, hi * sizeof(Scal), cudaMemcpyDeviceToHost, s->stream);
@@ -1110,6 +1197,7 @@ extern "C" pb_status pb_server_create(pb_ctx *ctx, size_t budget, const pb_solve
   s->ctx->stream = s->stream;
   s->ctx->own_stream = false;
   s->ctx->num_sms = ctx->num_sms;
+  s->ctx->max_smem = ctx->max_smem;
   s->ctx->stats = ctx->stats;
   ok = ok && cudaMallocHost((void **)&s->ctx->host_scal, sizeof(Scal) * 64) == cudaSuccess;
   ok = ok && !pb_dalloc((void **)&s->d_scal, MAX_SLOTS * sizeof(Scal));
@@ -1211,7 +1299,7 @@ extern "C" pb_status pb_server_destroy(pb_server *s) {
     }
   if (s->graph) cudaGraphExecDestroy(s->graph);
   void *ptrs[] = {s->d_scal, s->d_inst, s->d_counts, s->d_list, s->d_err, s->d_st,
-                  s->d_st_part, s->d_rs_part, s->d_rlist};
+                  s->d_st_part, s->d_rs_part, s->d_rlist, s->d_packets};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (s->h_scal) cudaFreeHost(s->h_scal);
