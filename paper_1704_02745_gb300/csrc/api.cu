@@ -85,6 +85,7 @@ extern "C" pb_status pb_create(pb_ctx **out, int device, void *cuda_stream) {
   }
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
   cudaDeviceGetAttribute(&c->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, device);
   if (cudaMallocHost((void **)&c->host_scal, sizeof(Scal) * 64) != cudaSuccess) {
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -793,7 +794,7 @@ static bool use_resident(pb_grid *g, const pb_solve_opts *o, int mode, int coef)
     g->res_mode = mode;
     g->res_coef = coef;
     g->res_fits = resident_plan(g->d.nx, g->d.ny, g->d.nz, mode, coef, g->ctx->num_sms,
-                                g->ctx->max_smem, &g->res_plan);
+                                g->ctx->max_smem, g->ctx->l2_bytes, &g->res_plan);
   }
   return g->res_fits;
 }

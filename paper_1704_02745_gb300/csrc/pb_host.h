@@ -16,6 +16,7 @@ struct pb_ctx {
   bool own_stream = false;
   int num_sms = 1;
   int max_smem = 0;  // shared memory a CTA may ask for, bytes
+  int l2_bytes = 0;
   pb::Scal *host_scal = nullptr;  // pinned, for convergence polls
   // pb_ctx_stats counters; a server's internal context counts into its parent's
   std::atomic<unsigned long long> launches{0}, h2d{0}, d2h{0};

@@ -1038,14 +1038,24 @@ ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &
 
 // The plan of least cost: of an iteration (alone), or of an iteration of as many
 // such grids as the device holds at once, a grid.
-static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, bool alone, ResPlan *out) {
+static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, long l2_bytes, bool alone,
+                      ResPlan *out) {
   const int es = mode == MODE_F64 ? 8 : 4, gpr = (nx + 3) / 4;
   const Build *builds = !alone ? BATCH_BUILDS : mode == MODE_F64 ? F64_BUILDS : F32_BUILDS;
   const int nb = !alone ? std::size(BATCH_BUILDS) : mode == MODE_F64 ? std::size(F64_BUILDS) : std::size(F32_BUILDS);
+  // What an FP32 iteration of the G = 0 builds reads of L2: the coefficients, z, d.
+  // More than 7/8 of L2 goes to memory in part, in the order of the bricks and
+  // twice, and the two-pass form is faster (L2 of 135 MB, FP32 coefficients, us an
+  // iteration in two passes -> here: 169^3, 116 MB, 72 -> 63; 173^3, 124 MB, 76 ->
+  // 84; 177^3, 133 MB, 81 -> 96; BF16: 177^3, 89 MB, 76 -> 66).  (FP64 waits for its
+  // arithmetic: 129^3 with explicit coefficients, 120 MB, 189 -> 148.)
+  const int coef_bytes = coef == COEF_PACKED ? 1 : coef == COEF_BF16 ? 8 : 16;
+  const bool in_l2 = mode == MODE_F64 || (long)nx * ny * nz * (coef_bytes + 8) <= l2_bytes / 8 * 7;
   bool found = false;
   double best = 0;
   for (int b = 0; b < nb; b++) {
     const Build &B = builds[b];
+    if (B.G == 0 && !in_l2) continue;
     const int per_sm = ctas_per_sm(B.threads), room = per_sm * num_sms;
     // (an SM keeps 1 KB of each CTA's shared memory to itself)
     const int smem = (max_smem + 1024) / per_sm - 1024 - RES_STATIC_SMEM / per_sm;
@@ -1086,11 +1096,11 @@ static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, i
   }
   return found;
 }
-bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, ResPlan *out) {
-  return best_plan(nx, ny, nz, mode, coef, num_sms, max_smem, true, out);
+bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, long l2_bytes, ResPlan *out) {
+  return best_plan(nx, ny, nz, mode, coef, num_sms, max_smem, l2_bytes, true, out);
 }
 bool resident_batch_plan(int nx, int ny, int nz, int num_sms, int max_smem, ResPlan *out) {
-  return best_plan(nx, ny, nz, MODE_F32_REFINE, COEF_PACKED, num_sms, max_smem, false, out);
+  return best_plan(nx, ny, nz, MODE_F32_REFINE, COEF_PACKED, num_sms, max_smem, 0, false, out);
 }
 
 size_t resident_packet_bytes(int ctas) { return 2 * PACKET_STRIDE * sizeof(Packet) * (size_t)ctas; }

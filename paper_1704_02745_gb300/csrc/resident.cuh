@@ -41,9 +41,9 @@ constexpr int RES_STATIC_SMEM = 16384;  // more than the kernel's static shared 
 constexpr int RES_MAX_PER_SM = 2;       // CTAs of a build on an SM at most
 
 // Plan of a grid for num_sms SMs of max_smem bytes a CTA (the largest one CTA
-// may ask for); false: the grid does
-// not fit (the two-pass form runs).
-bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, ResPlan *out);
+// may ask for) and l2_bytes of L2; false: it does not fit (the two-pass form
+// runs).
+bool resident_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, int max_smem, long l2_bytes, ResPlan *out);
 size_t resident_packet_bytes(int ctas);  // of a launch
 // Plan of a grid of a batch: for the most such grids at once (it does not depend
 // on what else runs, and so neither do the grid's sums).  FP32 with packed codes only.
