@@ -675,8 +675,7 @@ extern "C" pb_status pb_apply_operator(pb_grid *g, const void *u, void *au, int 
   Inst I;
   if ((st = pb_make_inst(g, nullptr, mode, pb_inner_coef(g, mode), I))) return st;
   cudaStream_t s = g->ctx->stream;
-  CK(cudaMemcpyAsync(g->dinst, &I, sizeof(Inst), cudaMemcpyHostToDevice, s));
-  CK(launch_apply(I, g->dinst, u, au, dtype == PB_F64 ? 0 : 1, s));
+  CK(launch_apply(I, u, au, dtype == PB_F64 ? 0 : 1, g->ctx->num_sms, s));
   g->ctx->stats->launches += 1;
   CK(cudaStreamSynchronize(s));
   return PB_OK;

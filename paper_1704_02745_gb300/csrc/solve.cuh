@@ -92,8 +92,7 @@ cudaError_t launch_pack(const double *dense, double *padded, int nx, int ny, int
                         cudaStream_t st);
 cudaError_t launch_unpack(const double *padded, double *dense, int nx, int ny, int nz, int px,
                           cudaStream_t st);
-cudaError_t launch_apply(const Inst &I, const Inst *dI, const void *u, void *au, int dtype,
-                         cudaStream_t st);
+cudaError_t launch_apply(const Inst &I, const void *u, void *au, int dtype, int num_sms, cudaStream_t st);
 // phi: nz x ny rows of px elements (px = nx: dense).  An atom whose
 // trilinear cell leaves the grid makes the energy NaN (periodic: corners wrap).
 cudaError_t launch_energy(const dbl4 *xyzq, int n_atoms, int nx, int ny, int nz, int px,
