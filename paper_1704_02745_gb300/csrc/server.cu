@@ -32,6 +32,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -143,7 +144,7 @@ struct Slot {
   Request req;
   bool warm = false;
   uint64_t first_round = 0;   // round whose graph first runs the current solve
-  Inst inst;                  // its descriptor, as last uploaded
+  std::unique_ptr<Inst> inst; // its descriptor, as last uploaded
   ResPlan res_plan;           // plan of its resident inner solves
   bool res_fits = false;
   bool ticked = false;        // phase ticks have run on the current solve: it may be inside an inner solve
@@ -494,7 +495,7 @@ bool rebuild_batch(pb_server *s, Stage &sg, bool *graph_stale) {
     if (pb_make_inst(g, &s->opts, s->mode, s->coef, I)) return false;
     I.s = s->d_scal + j;
     I.ap = nullptr;  // the update pass forms Ap again from p (k_update_tile)
-    s->slots[j].inst = I;
+    s->slots[j].inst.reset(new Inst(I));
     I.st_base = st_off;
     I.rs_base = rs_off;
     rs_off += g->n_rs;
@@ -637,7 +638,7 @@ bool run_resident_round(pb_server *s, std::vector<int> run, bool *ticks) {
     const int n = (int)l.slots.size();
     for (int k = 0; k < n; k++) {
       P[k] = &s->slots[l.slots[k]].res_plan;
-      I[k] = &s->slots[l.slots[k]].inst;
+      I[k] = s->slots[l.slots[k]].inst.get();
     }
     if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, s->stream) != cudaSuccess) {
       cudaGetLastError();  // ticks go on from the state the residual pass left
