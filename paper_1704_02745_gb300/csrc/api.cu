@@ -217,8 +217,12 @@ void pb_apply_plan(pb_grid *g, const KernelGrid &kg, bool batch, int tiles_x, in
   g->tiles_z = (nz + g->tz - 1) / g->tz;
   g->n_st = cols * g->tiles_z;
   // residual pass (FP64 arithmetic, not memory bound): pieces of RESID_TZ
-  // planes, so that even one grid's pass spreads over every SM
-  g->rtz = std::min(g->tz, RESID_TZ);
+  // planes, fewer on a single grid whose pieces then still run all at once
+  // (33^3: one plane, 36 -> 19 us; 65^3: 44 -> 34; a second wave costs more than
+  // shorter pieces give: 97^3 in 3 planes 46 -> 64)
+  g->rtz = 1;
+  while (g->rtz < RESID_TZ && (batch || cols * ((nz + g->rtz - 1) / g->rtz) > kg.resid_blocks)) g->rtz++;
+  g->rtz = std::min(g->tz, g->rtz);
   g->n_rs = cols * ((nz + g->rtz - 1) / g->rtz);
   // update chunks: one wave of resident update CTAs on large grids, never
   // fewer than CH elements per chunk
