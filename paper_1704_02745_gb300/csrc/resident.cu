@@ -196,9 +196,11 @@ __device__ __forceinline__ int load_error(const int *p) {
   asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-// Polls before a wait gives up: about 0.2 s of L2 round trips.  Counted in
-// polls, not in clock cycles, so that a preempted context does not time out.
-constexpr int RES_MAX_POLLS = 400000;
+// Polls before a wait gives up: about 4 s of L2 round trips, so that CTAs that got
+// their SMs outlast long kernels of other streams that still hold the others'.
+// Counted in polls, not in clock cycles, so that a preempted context does not
+// time out.
+constexpr int RES_MAX_POLLS = 8000000;
 
 #ifdef PB_FAULT_TEST
 // Test builds only: while positive, the first grid-wide wait of a CTA gives up.
