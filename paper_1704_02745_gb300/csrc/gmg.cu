@@ -1052,8 +1052,7 @@ static pb_status mg_build(pb_grid *g, pb_mg **out) {
     m->tail--;
     m->T = T;
   }
-  if (m->tail < m->lv.size() &&
-      cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, m->T.all * 4) != cudaSuccess) {
+  if (m->tail < m->lv.size() && allow_all_smem(k_mg_tail) != cudaSuccess) {
     cudaGetLastError();
     m->tail = m->lv.size();
   }

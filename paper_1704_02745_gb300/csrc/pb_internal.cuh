@@ -155,6 +155,19 @@ __host__ __device__ inline int dtab_index(uint32_t c) {
 }
 
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
+
+// Let a kernel ask for all the shared memory a CTA can have.  The limit belongs to the
+// kernel and is shared by every grid, context and thread of the process, so it is
+// never set to what one launch needs: that would refuse the larger launches of others.
+template <typename K> inline cudaError_t allow_all_smem(K *kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+}
 inline int pitch_of(int nx) { return round_up(nx + 1, PITCH_ALIGN); }
 
 }  // namespace pb

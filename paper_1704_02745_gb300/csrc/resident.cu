@@ -948,7 +948,7 @@ struct Shape {  // of a launch
 };
 template <typename W, typename K>
 cudaError_t launch_kernel(K *k, const Shape &P, const W &wave, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
+  const cudaError_t e = allow_all_smem(k);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.ctas);
