@@ -650,7 +650,10 @@ __global__ void __launch_bounds__(HARMONIC_NT)
     k -= 1;
     out = ez + ((size_t)(k + 1) * g.ny + j) * g.px + i;
   }
-  const float hf = (float)g.h, MARGIN = 1e-3f + 2e-6f * hf * (float)max(max(g.nx, g.ny), g.nz);
+  // Error of the FP32 test, u = 2^-24, L the grid's extent, R a radius: a coordinate
+  // relative to an atom is off by u (3 L + 2 R) at most near its sphere, and room = R^2
+  // - (fu^2 + fv^2) by u (9 R L + 13 R^2).  The margins are three times that and more.
+  const float hf = (float)g.h, L = hf * (float)max(max(g.nx, g.ny), g.nz), MARGIN = 1e-3f + 2e-6f * L;
   const float pf[3] = {(float)i * hf, (float)j * hf, (float)k * hf};
   // cells within r_max of the edge, in coordinates relative to the cells' corner
   // (o - h - cell size), widened by more than the FP32 error
@@ -700,7 +703,7 @@ __global__ void __launch_bounds__(HARMONIC_NT)
     hi_iv[at] = hi;
   };
   // FP32 test relative to the grid origin: the perpendicular distance and the
-  // extent along the axis, with a margin far above their FP32 error
+  // extent along the axis, each with its margin
   for (int cz = lo_c[2]; cz <= hi_c[2] && !full; cz++)
     for (int cy = lo_c[1]; cy <= hi_c[1] && !full; cy++) {
       // the cells of a row are neighbours in the list
@@ -710,11 +713,12 @@ __global__ void __launch_bounds__(HARMONIC_NT)
         const float rc[3] = {R.x, R.y, R.z};
         const float fu = pf[u] - rc[u], fv = pf[v] - rc[v], fa = rc[ax] - pf[ax];
         const float room = R.w * R.w - (fu * fu + fv * fv);
-        if (room < -MARGIN) continue;
-        if (fa + R.w < -MARGIN || fa - R.w > hf + MARGIN) continue;
-        if (room > MARGIN) {
-          const float q = sqrtf(room - MARGIN);
-          if (fa - q < -MARGIN && fa + q > hf + MARGIN) {
+        const float m_room = MARGIN + 2e-6f * R.w * (L + R.w), m_axis = MARGIN + 1e-6f * R.w;
+        if (room < -m_room) continue;
+        if (fa + R.w < -m_axis || fa - R.w > hf + m_axis) continue;
+        if (room > m_room) {
+          const float q = sqrtf(room - m_room);
+          if (fa - q < -m_axis && fa + q > hf + m_axis) {
             full = true;
             break;
           }
