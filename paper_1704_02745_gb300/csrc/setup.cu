@@ -233,8 +233,8 @@ __device__ __noinline__ double dh_term_any(double d2, double q, double kappa, do
   const double r = __dsqrt_rn(d2);
   return __ddiv_rn(__dmul_rn(q, exp(-__dmul_rn(kappa, r))), __dmul_rn(eps_out, r));
 }
-__device__ __forceinline__ bool dh_plain_range(double v) {  // 2^-120 <= |v| < 2^120
-  return (((uint32_t)__double2hiint(v) & 0x7fffffffu) - ((1023u - 120u) << 20)) < 240u << 20;
+template <uint32_t E> __device__ __forceinline__ bool dh_plain_range(double v) {  // 2^-E <= |v| < 2^E
+  return (((uint32_t)__double2hiint(v) & 0x7fffffffu) - ((1023u - E) << 20)) < 2 * E << 20;
 }
 // whether ghost node t is the first of its line (the fastest index of its face)
 __device__ __forceinline__ bool ghost_starts_line(const Geom &g, long t) {
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(DHX_NT) k_dh_f64(const dbl4 *xyzq, int n_atoms
   const double along = along_y ? py : px;
   const int axis = along_y ? 1 : 0;
   const double inv_eps = __drcp_rn(eps_out);
-  const bool eps_plain = dh_plain_range(eps_out);
+  const bool eps_plain = dh_plain_range<120>(eps_out);
   double s = 0.0;
   auto load = [&](int base) {
     if ((int)threadIdx.x < DHX_ATOMS && base + (int)threadIdx.x < n_atoms)
@@ -314,8 +314,11 @@ __global__ void __launch_bounds__(DHX_NT) k_dh_f64(const dbl4 *xyzq, int n_atoms
       const double tq = __dmul_rn(w, exp(-__dmul_rn(kappa, r))), b = __dmul_rn(eps_out, r);
       const double yi = __dmul_rn(y, inv_eps), q0 = __dmul_rn(tq, yi);
       v = fma(fma(-q0, b, tq), yi, q0);
-      // (tq = 0: v is 0 either way)
-      if (!(eps_plain && hi - ((1023u - 120u) << 20) < 240u << 20 && (dh_plain_range(tq) || dh_zero(tq))))
+      // d2 has to be a float; tq, whose quotient by b (2^+-180 at most) and remainder
+      // have to be normal numbers, may lie in 2^+-820: terms screened by less than
+      // e^-568, so that a long grid's far ones stay here too (3x3x20000 nodes with
+      // salt, whole setup: 2^+-120 for both 1,394 us, so 1,014; tq = 0: v is 0 either way)
+      if (!(eps_plain && hi - ((1023u - 120u) << 20) < 240u << 20 && (dh_plain_range<820>(tq) || dh_zero(tq))))
         v = dh_term_any(d2, w, kappa, eps_out);
       term[buf][u][lane] = v;
     }
