@@ -191,8 +191,10 @@ __device__ __forceinline__ void mg_pdl() {
 }
 
 // A thread's column: a group of four x nodes of row j, planes k0 .. k1 - 1.
-// Consecutive threads are consecutive groups whatever nx is, and one division
-// serves the column.
+// Consecutive threads are consecutive groups whatever nx is, on to the next run of
+// planes at a plane's end (a plane of 3x3 nodes has three groups: with CTAs that end
+// at a plane's end, 3x3x20000 nodes took 2,551 us a solve, so 689), and two
+// divisions serve the column.
 struct Column {
   uint32_t o;      // offset of the group in a plane
   int i, j, k0, k1;
@@ -201,12 +203,13 @@ struct Column {
 };
 __device__ __forceinline__ Column mg_column(const MgDims &d, int zc) {
   Column c;
-  const uint32_t gpr = (uint32_t)d.pitch() / 4, t = blockIdx.x * MG_NT + threadIdx.x;
-  c.in = t < gpr * (uint32_t)d.ny;
+  const uint32_t gpr = (uint32_t)d.pitch() / 4, groups = gpr * (uint32_t)d.ny, all = blockIdx.x * MG_NT + threadIdx.x;
+  const uint32_t run = all / groups, t = all - run * groups;
   c.j = (int)(t / gpr);
   c.i = 4 * (int)(t - (uint32_t)c.j * gpr);
   c.o = (uint32_t)c.j * (uint32_t)d.pitch() + (uint32_t)c.i;
-  c.k0 = blockIdx.y * zc;
+  c.in = run < (uint32_t)(d.nz + zc - 1) / (uint32_t)zc;
+  c.k0 = (int)run * zc;
   c.k1 = min(c.k0 + zc, d.nz);
   c.mask = c.i + 4 <= d.nx ? 0xFu : (1u << (d.nx - c.i)) - 1u;
   return c;
@@ -214,7 +217,7 @@ __device__ __forceinline__ Column mg_column(const MgDims &d, int zc) {
 // The launch of a column kernel over a level: planes of a column, and the grid.
 struct MgLaunch {
   int zc;
-  dim3 grid;
+  unsigned ctas;
 };
 // One wave of resident CTAs (a second, partly empty one costs as much as the
 // first: the FP64 operator at 129^3 in 1.2 waves took 44 us, in one 34), or
@@ -223,10 +226,10 @@ template <typename F>
 static MgLaunch mg_plan(F *kernel, const MgDims &d, int num_sms) {
   int per_sm = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, MG_NT, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-  const int cols = (int)(((size_t)d.pitch() / 4 * d.ny + MG_NT - 1) / MG_NT);
-  const int chunks = std::max(1, std::min(d.nz, num_sms * per_sm / cols));
-  const int zc = (d.nz + chunks - 1) / chunks;
-  return MgLaunch{zc, dim3((unsigned)cols, (unsigned)((d.nz + zc - 1) / zc))};
+  const size_t groups = (size_t)d.pitch() / 4 * d.ny;
+  const int runs = std::max(1, (int)std::min((size_t)d.nz, (size_t)num_sms * per_sm * MG_NT / groups));
+  const int zc = (d.nz + runs - 1) / runs;
+  return MgLaunch{zc, (unsigned)((groups * ((d.nz + zc - 1) / zc) + MG_NT - 1) / MG_NT)};
 }
 
 template <typename T> struct V4 { T v[4]; };
@@ -342,6 +345,8 @@ __device__ __forceinline__ void keep(V4<float> &a, uint32_t mask) {
 // bit of a scalar into 1e-8 of the solution to 1e-6 (the FP32 copy of r rounds
 // differently, and so on), so the order of these sums is part of the result.
 enum : int { DOT_ALPHA, DOT_STOP, DOT_BETA, DOT_RR };
+// Loads in flight a thread: half of the 33 nodes it has at 129^3, so two trips to
+// memory (with 8, five: an iteration 239 us for 218); a larger grid takes more trips.
 constexpr int MG_DOT_CTAS = 256, MG_DOT_BATCH = 17;
 __device__ __forceinline__ double mg_wide(double v) { return v; }
 __device__ __forceinline__ double mg_wide(float v) { return widen(v); }
@@ -355,6 +360,7 @@ __global__ void __launch_bounds__(MG_NT) k_mg_dot(MgDims d, MgScal *S, const dou
   const uint32_t lo = blockIdx.x * per, hi = min(lo + per, n);
   uint32_t t = lo + threadIdx.x;
   uint32_t row = t / nx, i = t - row * nx;
+  const uint32_t rows = MG_NT / nx, rest = MG_NT - rows * nx;  // MG_NT nodes on
   double s = 0.0;
   while (t < hi) {
     double u[MG_DOT_BATCH];
@@ -369,8 +375,9 @@ __global__ void __launch_bounds__(MG_NT) k_mg_dot(MgDims d, MgScal *S, const dou
         m++;
       }
       t += MG_NT;
-      i += MG_NT;
-      while (i >= nx) {
+      i += rest;
+      row += rows;
+      if (i >= nx) {
         i -= nx;
         row++;
       }
@@ -1169,7 +1176,7 @@ template <typename A0, typename... Params, typename... Args>
 static void mg_columns(const pb_mg *m, const MgDims &d, cudaStream_t s, unsigned long long &launches,
                        void (*k)(A0, int, Params...), const A0 &a0, Args... args) {
   const MgLaunch L = mg_plan(k, d, m->num_sms);
-  mg_launch(k, L.grid, MG_NT, 0, s, a0, L.zc, args...);
+  mg_launch(k, dim3(L.ctas), MG_NT, 0, s, a0, L.zc, args...);
   launches++;
 }
 // ... of the two builds by operator storage
