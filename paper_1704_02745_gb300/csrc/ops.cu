@@ -47,8 +47,9 @@ cudaError_t launch_unpack(const double *padded, double *dense, int nx, int ny, i
 // (A u)_c = diag_c u_c - sum_nb eps_edge u_nb, ghosts zero; dense u and Au.
 // Bound by the call on small grids (the descriptor travels as a kernel argument:
 // uploading it first cost more than the kernel), by FP64 arithmetic or DRAM on
-// large ones: a thread walks kz nodes of a z column, so that the index division
-// is one a column and u is read five times a node instead of seven.  Measured, a
+// large ones: a thread walks kz nodes of a z column, so that the index divisions
+// are two a column and u is read five times a node instead of seven; CTAs run on
+// into the next planes at a plane's end (3x3x20000 nodes, FP64, 34 -> 24 us).  Measured, a
 // call, against the uploaded descriptor and one node a thread: 33^3 14.5 -> 12.7 us;
 // 257^3 FP64 218 -> 216, FP32 packed 94 -> 77, BF16 112 -> 94, FP32 109 -> 97 (packed:
 // kz = 16 and 1 94 and 133; explicit storage: two nodes in flight 110 .. 138).  Six
@@ -59,50 +60,50 @@ __global__ void __launch_bounds__(256, 6) k_apply(const __grid_constant__ Inst I
                                                   T *__restrict__ au, int kz) {
   constexpr int UNROLL = CM == COEF_PACKED ? 2 : 1;
   const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const uint32_t plane = (uint32_t)nx * ny, p = blockIdx.x * 256u + threadIdx.x;
-  if (p >= plane) return;
+  const uint32_t plane = (uint32_t)nx * ny, t = blockIdx.x * 256u + threadIdx.x;
+  const uint32_t run = t / plane, p = t - run * plane;  // run of kz planes, place in a plane
+  const long k0 = (long)run * kz;
+  if (k0 >= nz) return;
   const int j = (int)(p / (uint32_t)nx), i = (int)(p - (uint32_t)j * nx);
   const bool per = I.periodic != 0;
   // offsets of the in-plane neighbours (with wrap: modulo n)
   const long xm = i > 0 ? -1 : nx - 1, xp = i < nx - 1 ? 1 : 1 - nx;
   const long ym = j > 0 ? -nx : (long)plane - nx, yp = j < ny - 1 ? nx : nx - (long)plane;
   const bool has_xm = per || i > 0, has_xp = per || i < nx - 1, has_ym = per || j > 0, has_yp = per || j < ny - 1;
-  for (long k0 = (long)blockIdx.y * kz; k0 < nz; k0 += (long)gridDim.y * kz) {
-    const int k1 = (int)(k0 + kz < nz ? k0 + kz : nz);
-    const T *uk = u + (size_t)k0 * plane + p;
-    T *ak = au + (size_t)k0 * plane + p;
-    size_t e = ((size_t)k0 * ny + j) * I.px + i;
-    T below = 0, here = *uk;
-    if (k0 > 0) below = uk[-(long)plane];
-    else if (per) below = u[(size_t)(nz - 1) * plane + p];
+  const int k1 = (int)(k0 + kz < nz ? k0 + kz : nz);
+  const T *uk = u + (size_t)k0 * plane + p;
+  T *ak = au + (size_t)k0 * plane + p;
+  size_t e = ((size_t)k0 * ny + j) * I.px + i;
+  T below = 0, here = *uk;
+  if (k0 > 0) below = uk[-(long)plane];
+  else if (per) below = u[(size_t)(nz - 1) * plane + p];
 #pragma unroll UNROLL
-    for (int k = (int)k0; k < k1; k++) {
-      T above = 0;
-      if (k < nz - 1) above = uk[plane];
-      else if (per) above = u[p];
-      const NodeCoef<T> c = node_coef<T, CM>(I, e, k);
-      T s = 0;
-      if (has_xm) s += c.exm * uk[xm];
-      if (has_xp) s += c.exp * uk[xp];
-      if (has_ym) s += c.eym * uk[ym];
-      if (has_yp) s += c.eyp * uk[yp];
-      if (per || k > 0) s += c.ezm * below;
-      if (per || k < nz - 1) s += c.ezp * above;
-      *ak = c.diag * here - s;
-      below = here;
-      here = above;
-      uk += plane;
-      ak += plane;
-      e += (size_t)I.px * ny;
-    }
+  for (int k = (int)k0; k < k1; k++) {
+    T above = 0;
+    if (k < nz - 1) above = uk[plane];
+    else if (per) above = u[p];
+    const NodeCoef<T> c = node_coef<T, CM>(I, e, k);
+    T s = 0;
+    if (has_xm) s += c.exm * uk[xm];
+    if (has_xp) s += c.exp * uk[xp];
+    if (has_ym) s += c.eym * uk[ym];
+    if (has_yp) s += c.eyp * uk[yp];
+    if (per || k > 0) s += c.ezm * below;
+    if (per || k < nz - 1) s += c.ezp * above;
+    *ak = c.diag * here - s;
+    below = here;
+    here = above;
+    uk += plane;
+    ak += plane;
+    e += (size_t)I.px * ny;
   }
 }
 
 cudaError_t launch_apply(const Inst &I, const void *u, void *au, int dtype, int num_sms, cudaStream_t st) {
   // columns of up to 4 nodes while that leaves eight CTAs an SM and more
-  const long cols = ((long)I.nx * I.ny + 255) / 256;
-  const int kz = (int)std::max(1l, std::min(4l, cols * I.nz / (16l * num_sms)));
-  const dim3 blocks((unsigned)cols, (unsigned)std::min(65535, (I.nz + kz - 1) / kz));
+  const long plane = (long)I.nx * I.ny;
+  const int kz = (int)std::max(1l, std::min(4l, plane * I.nz / (256l * 16l * num_sms)));
+  const unsigned blocks = (unsigned)((plane * ((I.nz + kz - 1) / kz) + 255) / 256);
   if (dtype == 0) {  // FP64: exact coefficients
     if (I.coef == COEF_F64)
       k_apply<double, COEF_F64><<<blocks, 256, 0, st>>>(I, (const double *)u, (double *)au, kz);
