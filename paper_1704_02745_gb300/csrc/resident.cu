@@ -1053,6 +1053,14 @@ static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, i
   // arithmetic: 129^3 with explicit coefficients, 120 MB, 189 -> 148.)
   const int coef_bytes = coef == COEF_PACKED ? 1 : coef == COEF_BF16 ? 8 : 16;
   const bool in_l2 = mode == MODE_F64 || (long)nx * ny * nz * (coef_bytes + 8) <= l2_bytes / 8 * 7;
+  // Explicit coefficients in the G = 0 builds: a plane waits for its loads, and a narrow,
+  // deep brick has few warps to wait beside each other.  The two-pass form is faster
+  // beyond these planes at these warps (us an iteration in two passes -> here: FP32
+  // 17x17x1976, 13 planes, 34.6 -> 34.6, x2432, 16, 36.5 -> 44.3, 25x25x2432, 6 warps,
+  // 45.9 -> 47.8, 9x65x2432, 7 warps, 58 -> 48; BF16 17x17x2432 37.0 -> 38.8, x2888, 19,
+  // 40 -> 46; FP64 9x9x1976 82 -> 79, x2432 87 -> 97.  Packed codes: faster at any).
+  const int few_warps = coef == COEF_F32 ? 6 : coef == COEF_BF16 ? 5 : coef == COEF_F64 ? 4 : 0;
+  const int deep = coef == COEF_BF16 ? 16 : 13;
   bool found = false;
   double best = 0;
   for (int b = 0; b < nb; b++) {
@@ -1073,6 +1081,7 @@ static bool best_plan(int nx, int ny, int nz, int mode, int coef, int num_sms, i
         P.gpr = gpr;
         P.threads = std::max(128, (P.by * gpr + 31) / 32 * 32);  // four warps: grid_sum
         if (P.threads > B.threads || P.bz > 32 || 2 * P.bz * gpr > RES_YH * P.threads) continue;
+        if (B.G == 0 && P.threads <= 32 * few_warps && P.bz > deep) continue;
         P.off_ap = (int)p_bytes(P.by, P.bz, gpr, es);
         // (in a batch the launch has the threads of its largest plan)
         if ((long)smem_of(P, es, coef, alone ? P.threads : B.threads) > smem) continue;
