@@ -786,7 +786,8 @@ pb_status pb_run_ticks(pb_grid *g, int mode, int coef, int ticks) {
 // ms) to 187x161x175 (13.6 -> 8.9 ms), the largest it holds in FP32, and for
 // FP64 at 129^3 (40 -> 22 ms).  pb_solve_opts.poll_every and profile ask for
 // the tick form, whose passes they count; it also serves a grid whose
-// cooperative launch the device refuses.
+// cooperative launch the device refuses, and a solve whose CTAs do not all come
+// to run within the limit of the resident form's waits (about 4 s).
 static bool use_resident(pb_grid *g, const pb_solve_opts *o, int mode, int coef) {
   if (o->profile || o->poll_every > 0) return false;
   if (g->res_mode != mode || g->res_coef != coef) {
@@ -1037,18 +1038,24 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
   if ((st = pb_make_inst(g, &oo, mode, coef, I))) return st;
   if (grid_tile_update(g, mode, coef)) I.ap = nullptr;  // the update pass forms Ap again
   Scal S0 = pb_initial_scal(g->bnorm);
-  CK(cudaMemsetAsync(g->err, 0, sizeof(int) * 4, s));
   CK(cudaMemcpyAsync(g->dinst, &I, sizeof(Inst), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g->scal, &S0, sizeof(Scal), cudaMemcpyHostToDevice, s));
-  static const int one_pending = 1;  // the solve opens with a residual pass
-  CK(cudaMemcpyAsync(g->counts + 2, &one_pending, sizeof(int), cudaMemcpyHostToDevice, s));
-  g->ctx->stats->h2d += sizeof(Inst) + sizeof(Scal) + sizeof(int);
-  if (o->warm_start) {
-    CK(launch_pack(phi, g->x64, g->d.nx, g->d.ny, g->d.nz, g->g.px, s));
-    g->ctx->stats->launches += 1;
-  } else {
-    CK(cudaMemsetAsync(g->x64, 0, g->n_pad * sizeof(double), s));
-  }
+  g->ctx->stats->h2d += sizeof(Inst);
+  // scalars, error word and x as a solve finds them (phi is written at its end only)
+  auto start = [&]() -> pb_status {
+    CK(cudaMemsetAsync(g->err, 0, sizeof(int) * 4, s));
+    CK(cudaMemcpyAsync(g->scal, &S0, sizeof(Scal), cudaMemcpyHostToDevice, s));
+    static const int one_pending = 1;  // the solve opens with a residual pass
+    CK(cudaMemcpyAsync(g->counts + 2, &one_pending, sizeof(int), cudaMemcpyHostToDevice, s));
+    g->ctx->stats->h2d += sizeof(Scal) + sizeof(int);
+    if (o->warm_start) {
+      CK(launch_pack(phi, g->x64, g->d.nx, g->d.ny, g->d.nz, g->g.px, s));
+      g->ctx->stats->launches += 1;
+    } else {
+      CK(cudaMemsetAsync(g->x64, 0, g->n_pad * sizeof(double), s));
+    }
+    return PB_OK;
+  };
+  if ((st = start())) return st;
   const int ticks = o->poll_every > 0 ? o->poll_every : auto_ticks(g);
   // every tick advances at least one phase step; bound the host loop
   const long max_ticks = (long)oo.max_iter + 2L * (oo.max_outer + 2) + 4L * ticks;
@@ -1060,9 +1067,14 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
   } else {
     int *herr_poll = (int *)(hs + 1);  // pinned slot after the scalars
     for (;;) {
-      if (resident && run_resident(g, I, mode, coef) != cudaSuccess) {
-        cudaGetLastError();  // the tick form goes on from the same state
-        resident = g->res_fits = false;
+      if (resident) {
+        const cudaError_t e = run_resident(g, I, mode, coef);
+        if (e != cudaSuccess) {
+          cudaGetLastError();  // the tick form goes on from the same state
+          resident = false;
+          // memory may be free again by the next solve; any other refusal stands
+          if (e != cudaErrorMemoryAllocation) g->res_fits = false;
+        }
       }
       if (!resident && (st = pb_run_ticks(g, mode, coef, ticks))) return st;
       done_ticks += resident ? 1 : ticks;  // (a resident graph advances by an inner solve at least)
@@ -1070,8 +1082,16 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
       CK(cudaMemcpyAsync(herr_poll, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
       g->ctx->stats->d2h += sizeof(Scal) + sizeof(int);
       CK(cudaStreamSynchronize(s));
+      if (*herr_poll & ERR_RESIDENT) {
+        // The CTAs of an inner solve did not all come to run within its waits' limit (other
+        // work held their SMs), and left its vectors in pieces: over again, in ticks.
+        if ((st = start())) return st;
+        resident = false;
+        done_ticks = 0;
+        continue;
+      }
       if (hs->phase == PH_DONE) break;
-      if (*herr_poll & 2) break;  // a pipeline wait gave up: the solve cannot finish
+      if (*herr_poll & ERR_WAIT) break;  // a pipeline wait gave up: the solve cannot finish
       if (done_ticks > max_ticks) {
         hs->status = PB_ERR_TIMEOUT;
         break;
@@ -1083,7 +1103,7 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
     int *herr = (int *)(hs + 1);  // pinned slot after the scalars
     CK(cudaMemcpyAsync(herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    if (*herr & 2) S.status = PB_ERR_TIMEOUT;  // a device pipeline wait gave up
+    if (*herr & ERR_WAIT) S.status = PB_ERR_TIMEOUT;  // a device pipeline wait gave up
   }
   CK(launch_unpack(S.xbuf ? g->x64b : g->x64, phi, g->d.nx, g->d.ny, g->d.nz, g->g.px, s));
   g->ctx->stats->launches += 1;

@@ -28,7 +28,8 @@
 //     Measured with 152 CTAs: 1,830 cycles (words side by side 4,060; pushed to
 //     152 mailboxes 2,800; through a master CTA 2,600; clusters of 4 and their
 //     leaders 3,900).  Polls are bounded: a CTA that gives up sets the error
-//     word and the others leave on seeing it.
+//     word, the others leave on seeing it, and the host starts the solve over in
+//     phase ticks, which need no CTA to run beside another.
 //   - the scalars stay off the FP64 pipe in FP32 solves (a warp's FP64 add takes
 //     19 cycles of an SM, a division 2,270 over 16 warps): sums and quotients
 //     are unevaluated pairs of floats (48 bits and more).
@@ -228,7 +229,7 @@ __device__ __forceinline__ bool await_word(const Packet *words, int c, Sum<T> (&
 #pragma unroll 1
   while (!wire_load(words + (size_t)PACKET_STRIDE * c, x, epoch)) {
     ++polls;
-    if (polls >= RES_MAX_POLLS || ((polls & 255) == 0 && (load_error(err) & 2))) return false;
+    if (polls >= RES_MAX_POLLS || ((polls & 255) == 0 && (load_error(err) & ERR_RESIDENT))) return false;
   }
   return true;
 }
@@ -297,7 +298,7 @@ __device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, int cta, int
     }
   }
   if (!ok) {
-    atomicOr(err, 2);
+    atomicOr(err, ERR_RESIDENT);
     S.failed = 1;
   }
   __syncthreads();
@@ -1157,7 +1158,7 @@ cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *co
 
 #ifdef PB_FAULT_TEST
 // Test builds only: see g_fault_abandon_sums.
-int pb_resident_abandon_sums(int count) {
+extern "C" int pb_test_abandon_sums(int count) {
   return cudaMemcpyToSymbol(pb::g_fault_abandon_sums, &count, sizeof(int)) == cudaSuccess ? 0 : 3;
 }
 #endif

@@ -1088,7 +1088,7 @@ void worker_main(pb_server *s) {
     }
     if (prev_graph) {
       if (!cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) break;
-      if (sp.counts[2] & 2) {
+      if (sp.counts[2] & (ERR_WAIT | ERR_RESIDENT)) {
         // A pipeline wait gave up in that graph (bounded device wait): the
         // grid whose tile was abandoned can no longer finish, and the error
         // word does not say which.  Fail every solve on the device with

@@ -985,7 +985,7 @@ __device__ __forceinline__ void cg_pass(const Batch &B) {
         cg_tile<T, CM, NS, PASS>(I, S, item.tile, stages, ring, dtab, mtab, full, SR, abort, v0, v1);
       }
       if (abort) {
-        if (threadIdx.x == 0) atomicOr(B.error, 2);  // a pipeline wait timed out
+        if (threadIdx.x == 0) atomicOr(B.error, ERR_WAIT);  // a pipeline wait timed out
         break;
       }
       if (threadIdx.x == 0) s_item = take_item(next);
@@ -1402,10 +1402,10 @@ KernelGrid kernel_grid(int mode, int coef, int num_sms, bool single) {
 #ifdef PB_FAULT_TEST
 // Test builds only: make the next `count` first-plane stage waits give up at
 // once (see g_fault_abandon_waits), and the next `count` first grid-wide sums
-// of the resident solve.  Returns 0, or PB_ERR_CUDA.
-int pb_resident_abandon_sums(int count);  // resident.cu
+// of the resident solve (pb_test_abandon_sums: those alone).  Returns 0, or PB_ERR_CUDA.
+extern "C" int pb_test_abandon_sums(int count);  // resident.cu
 extern "C" int pb_test_abandon_waits(int count) {
-  if (pb_resident_abandon_sums(count)) return 3;
+  if (pb_test_abandon_sums(count)) return 3;
   return cudaMemcpyToSymbol(pb::g_fault_abandon_waits, &count, sizeof(int)) == cudaSuccess ? 0 : 3;
 }
 #endif
