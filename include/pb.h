@@ -334,7 +334,10 @@ typedef struct {
  * admitted while the sum of pb_grid_bytes stays within it) and the solve
  * options applied to every request (precision, preconditioner, tolerances;
  * warm_start = 1: later snapshots of a trajectory start from its last
- * solution).  NULL opts: FP32 + FP64 refinement, Jacobi, rel_tol 1e-6.  The
+ * solution).  NULL opts: FP32 + FP64 refinement, Jacobi, rel_tol 1e-6.  A grid
+ * that registers and shared memory of the chip can hold is solved there, in whole
+ * inner solves, any other in phase ticks, whatever else runs beside it;
+ * poll_every > 0: all in ticks.  The
  * server runs a worker thread; pb_server_destroy stops it and frees all.
  * Failures reach the requests they concern, and the server goes on serving:
  * a grid the device has no memory for (after idle grids are released and the

@@ -15,10 +15,11 @@
 //      stencil tiles of every active grid, largest first, each grid's partial
 //      sums at its own offset, so its reductions are summed in a fixed order
 //      whatever else runs;
-//   4. queues whole inner solves of the batch's grids, kept on the chip
-//      (run_resident_round), or else a captured device graph of `ticks` phase
-//      ticks over the whole batch (finished grids are skipped by their
-//      convergence mask), and a copy of all grids' scalars;
+//   4. queues a captured device graph of `ticks` phase ticks over the grids that
+//      run in ticks (finished ones are skipped by their convergence mask), whole
+//      inner solves of the grids that stay on the chip (run_resident_round), and
+//      a copy of all grids' scalars;  a grid's form follows from its own size, so
+//      its result is the same whatever else runs;
 //   5. while that graph runs, reads the scalars the previous round's graph
 //      left, queues the energy (and phi) of the solves that finished in it on
 //      the copy stream, beside the running graph, and hands out the results
@@ -146,8 +147,8 @@ struct Slot {
   uint64_t first_round = 0;   // round whose graph first runs the current solve
   std::unique_ptr<Inst> inst; // its descriptor, as last uploaded
   ResPlan res_plan;           // plan of its resident inner solves
-  bool res_fits = false;
-  bool ticked = false;        // phase ticks have run on the current solve: it may be inside an inner solve
+  bool res_fits = false;      // it has one: its solves run in the resident form
+  bool ticked = false;        // the current solve runs in phase ticks all the same
 };
 
 // A finished solve whose energy (and phi) are queued behind the running graph.
@@ -384,7 +385,7 @@ std::vector<int> admit(pb_server *s) {
       cudaEventRecord(s->ev_idle[j], s->stream);  // its workspace clears
       cudaEventRecord(s->ev_energy[j], s->stream);
       Slot &sl = s->slots[j];
-      sl.res_fits = s->mode != MODE_F64 && s->coef == COEF_PACKED &&
+      sl.res_fits = s->mode != MODE_F64 && s->coef == COEF_PACKED && s->opts.poll_every <= 0 &&
                     resident_batch_plan(g->d.nx, g->d.ny, g->d.nz, s->ctx->num_sms, s->ctx->max_smem,
                                         &sl.res_plan);
       sl.g = g;
@@ -467,7 +468,6 @@ void replan_all(pb_server *s) {
     if (sl.g) pb_batch_plan_grid(sl.g, s->kg, s->plan.min_planes, s->plan.height_pct);
 }
 
-// Upload the descriptors, work lists and partial offsets of the active grids.
 // Host staging capacity for n items (pinned; the set is idle when called).
 bool stage_items(Stage &st, size_t n) {
   if (n <= st.cap_items) return true;
@@ -483,12 +483,20 @@ bool stage_items(Stage &st, size_t n) {
   return true;
 }
 
+// Whether a slot's current solve runs as whole inner solves on the chip
+// (run_resident_round) or in phase ticks.
+bool in_resident_form(const pb_server *s, const Slot &sl) {
+  return sl.res_fits && !sl.ticked && !s->resident_off;
+}
+
 bool rebuild_batch(pb_server *s, Stage &sg, bool *graph_stale) {
   std::vector<Item> st;
   std::vector<int> active;
   for (int j = 0; j < (int)s->slots.size(); j++)
     if (s->slots[j].g && s->slots[j].busy && !s->slots[j].pending) active.push_back(j);
   int st_off = 0, rs_off = 0, hi = 0;
+  // the fast builds of the tile passes serve ticks over no grid that wraps
+  bool fast = s->mode != MODE_F64 && s->coef == COEF_PACKED;
   for (int j : active) {
     pb_grid *g = s->slots[j].g;
     Inst &I = sg.inst[j];
@@ -499,13 +507,12 @@ bool rebuild_batch(pb_server *s, Stage &sg, bool *graph_stale) {
     I.st_base = st_off;
     I.rs_base = rs_off;
     rs_off += g->n_rs;
+    hi = j + 1;
+    if (in_resident_form(s, s->slots[j])) continue;  // residual passes only
     for (int t = 0; t < g->n_st; t++) st.push_back(Item{j, t});
     st_off += g->n_st;
-    hi = j + 1;
+    fast = fast && !g->d.periodic;
   }
-  // the fast builds of the tile passes serve a batch with no grid that wraps
-  bool fast = s->mode != MODE_F64 && s->coef == COEF_PACKED;
-  for (int j : active) fast = fast && !s->slots[j].g->d.periodic;
   if (s->kg.fast != (fast ? 1 : 0)) {
     s->kg.fast = fast ? 1 : 0;
     *graph_stale = true;
@@ -583,33 +590,25 @@ Batch server_batch(const pb_server *s) {
   return B;
 }
 
-// A round of whole inner solves instead of ticks: every grid of the batch has
-// a plan that keeps it on the chip, and none is inside an inner solve of ticks.
-// The grids run side by side, several to a cooperative launch, each on the SMs
-// its plan asks for; finished ones take none (the host reads the last round's
-// phases first, some tens of us in rounds of milliseconds).  Ticks are bound by
-// their bytes while many grids run and by latency when few are left; this form
-// by a CTA's chain of latencies, of which two CTAs an SM hide half.  Measured,
-// bursts to 1e-9, ticks -> here: one grid of 97^3 32.4 -> 3.9 ms; 32 of 49^3
-// 35.3 -> 10.6, of 97^3 98.8 -> 70.3, of 113^3 143 -> 139, of 129^3 204 -> 167;
-// 256 of 65^3 200 -> 133; 32 with wrap of 97x81x113 284 -> 93.  A batch with a
-// grid that does not fit (some 2.5 M nodes) runs in ticks: as many bytes a
-// second as this form needs for its share, and no grid waits for another.
-bool can_run_resident(const pb_server *s, const std::vector<int> &active) {
-  if (s->resident_off || s->mode == MODE_F64) return false;
-  for (int j : active)
-    if (!s->slots[j].res_fits || s->slots[j].ticked) return false;
-  return true;
-}
+// A round of whole inner solves: the grids whose plan keeps them on the chip run
+// side by side, several to a cooperative launch, each on the SMs its plan asks
+// for; finished ones take none (the host reads the last round's phases first,
+// while the round's ticks, if there are any, run).  Ticks are bound by their bytes
+// while many grids run and by latency when few are left; this form by a CTA's
+// chain of latencies, of which two CTAs an SM hide half.  Measured, bursts to
+// 1e-9, ticks -> here: one grid of 97^3 32.4 -> 3.9 ms; 32 of 49^3 35.3 -> 10.6,
+// of 97^3 98.8 -> 70.3, of 113^3 143 -> 139, of 129^3 204 -> 167; 256 of 65^3 200 ->
+// 133; 32 with wrap of 97x81x113 284 -> 93.  Grids too large for it (some 2.5 M
+// nodes), FP64 and servers created with poll_every > 0 run in ticks.
 
 // The residual pass, an inner solve of each grid of `run`, the residual pass.
-// ticks: nothing ran (the device refused the launch), ticks have to.
-bool run_resident_round(pb_server *s, std::vector<int> run, bool *ticks) {
-  *ticks = false;
+// *refused: the device refused a launch; ticks go on from the state as it stands.
+bool run_resident_round(pb_server *s, std::vector<int> run, bool *refused) {
+  *refused = false;
   const Batch B = server_batch(s);
   const size_t bytes = resident_packet_bytes(RES_MAX_PER_SM * s->ctx->num_sms);
   if (!s->d_packets && pb_dalloc(&s->d_packets, bytes)) {
-    s->resident_off = *ticks = true;
+    *refused = true;
     return true;
   }
   if (!cuda_ok(launch_phase(B, s->mode, s->coef, s->kg, 4, s->stream), s, "residual pass")) return false;
@@ -641,8 +640,8 @@ bool run_resident_round(pb_server *s, std::vector<int> run, bool *ticks) {
       I[k] = s->slots[l.slots[k]].inst.get();
     }
     if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, s->stream) != cudaSuccess) {
-      cudaGetLastError();  // ticks go on from the state the residual pass left
-      s->resident_off = *ticks = true;
+      cudaGetLastError();
+      *refused = true;
       return true;
     }
   }
@@ -1003,6 +1002,14 @@ void worker_main(pb_server *s) {
         }
       }
     }
+    // While kernels are measured every solve runs in the ticks that are measured.
+    const bool profiling = s->profiling.load();
+    if (profiling)
+      for (Slot &sl : s->slots)
+        if (sl.g && sl.busy && !sl.pending && in_resident_form(s, sl)) {
+          sl.ticked = true;
+          active_changed = true;
+        }
     if (!started.empty()) active_changed = true;
     if (active_changed) {
       // descriptors first: the start kernel reads each grid's error word and
@@ -1049,28 +1056,32 @@ void worker_main(pb_server *s) {
       if (!active.empty() && !rebuild_batch(s, sg, &graph_stale)) break;
     }
     if (want_tune) {
-      for (int j : active) s->slots[j].ticked = true;
+      for (int j : active) s->slots[j].ticked = true;  // the passes are timed on live solves
       if (!tune_batch(s, sg, active, &graph_stale)) break;
       if (!rebuild_batch(s, sg, &graph_stale)) break;
     }
     bool ran = false;
     if (!active.empty()) {
-      bool ticks = s->profiling.load() || !can_run_resident(s, active);
-      if (!ticks) {
+      std::vector<int> chip;
+      for (int j : active)
+        if (in_resident_form(s, s->slots[j])) chip.push_back(j);
+      if (profiling) {
+        if (!run_profiled(s, active, s->prof, s->ticks)) break;
+      } else if (chip.size() < active.size()) {
+        if (!run_graph(s, graph_stale)) break;
+        graph_stale = false;
+      }
+      if (!chip.empty()) {
         // what the last round left: grids that finished in it take no SMs
         if (prev_graph && !cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) break;
         std::vector<int> run;
-        for (int j : active)
+        for (int j : chip)
           if (s->slots[j].first_round == s->round || !prev_graph || sp.scal[j].phase != PH_DONE) run.push_back(j);
-        if (!run_resident_round(s, run, &ticks)) break;
-      }
-      if (ticks) {
-        for (int j : active) s->slots[j].ticked = true;
-        if (s->profiling.load()) {
-          if (!run_profiled(s, active, s->prof, s->ticks)) break;
-        } else {
-          if (!run_graph(s, graph_stale)) break;
-          graph_stale = false;
+        bool refused = false;
+        if (!run.empty() && !run_resident_round(s, run, &refused)) break;
+        if (refused) {
+          s->resident_off = true;
+          active_changed = true;
         }
       }
       const int hi = *std::max_element(active.begin(), active.end()) + 1;
