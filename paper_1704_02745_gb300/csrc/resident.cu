@@ -514,6 +514,27 @@ constexpr int RES_YH = 3;  // y-halo groups a thread can own
 // the other waits for its sums
 constexpr int ctas_per_sm(int threads) { return threads <= 256 ? 2 : 1; }
 
+// The direction p (array gp) of a CTA's brick into ps: rows -1 .. rows of planes -1 .. kn,
+// as an earlier launch left them.  Out of line: inlined, it took registers from the
+// iterations (spills of the 8-plane build 64 -> 92 bytes; a burst of 129^3 167 -> 177 ms).
+template <typename T, bool PER>
+__device__ __noinline__ void load_direction(const ResArgs &R, const T *gp, int cta, T *ps) {
+  const int gpr = R.gpr, by = R.by, ny = R.ny, nz = R.nz, rp = 4 * gpr + 4;
+  const int cy = cta % R.nby, y0 = cy * by, z0 = cta / R.nby * R.bz;
+  const int rows = min(by, ny - y0) + 2, planes = min(R.bz, nz - z0) + 2;
+  for (int f = threadIdx.x; f < planes * rows * gpr; f += blockDim.x) {
+    const int row = f / gpr, x = f - row * gpr, pl = row / rows, r = row - pl * rows;
+    int j = y0 + r - 1, k = z0 + pl - 1;
+    if (PER) {
+      j = j < 0 ? ny - 1 : j == ny ? 0 : j;
+      k = k < 0 ? nz - 1 : k == nz ? 0 : k;
+    }
+    if (j >= 0 && j < ny && k >= 0 && k < nz)
+      q_store(ps + (pl * (by + 2) + r) * rp + 4 + 4 * x,
+              q_load_l2(gp + ((uint32_t)k * ny + j) * R.px + 4 * x));
+  }
+}
+
 template <typename T, int CM, int G, int NTH, bool PER, typename W>
 __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __grid_constant__ W wave) {
   int n_grid = 0, cta = blockIdx.x, ncta = gridDim.x;  // this CTA's grid, its number there
@@ -533,7 +554,10 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
   __shared__ CodeEntry<T> mtab[CM == COEF_PACKED ? 128 : 1];
   const Inst &I = *R.inst;
   Scal *Sp = I.s;
-  if (*(volatile int *)&Sp->phase != PH_START) return;  // nothing to solve (the same for every CTA)
+  const int was = *(volatile int *)&Sp->phase;
+  constexpr bool ROUNDS = std::is_same_v<W, ResWave>;  // leaves a solve after `budget` iterations
+  if (was != PH_START && !(ROUNDS && was == PH_INNER)) return;  // nothing to solve (the same for every CTA)
+  const bool resume = ROUNDS && was == PH_INNER;  // goes on where an earlier launch left it
   if (threadIdx.x == 0) S.failed = 0;
   const int by = R.by, gpr = R.gpr, rp = 4 * gpr + 4, ps_plane = (by + 2) * rp;
   const int cy = cta % R.nby, cz = cta / R.nby;
@@ -604,6 +628,10 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
     S.neighbour[3] = cz < nbz - 1 ? b + nby : PER ? b - (nbz - 1) * nby : -1;
   }
 
+  if (resume) {
+    __syncthreads();  // ps is zero
+    load_direction<T, PER>(R, (const T *)(Sp->pbuf ? R.p1 : R.p0), cta, ps);
+  }
   const Q4<T> zero4 = dup4((T)0);
   Q4<T> z[REG ? G : 1], d[REG ? G : 1];
   if constexpr (REG) {
@@ -612,7 +640,7 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
       z[k] = d[k] = zero4;
       if (own && k < kn) {
         z[k] = q_load_l2(gz + e0 + k * plane);
-        if (!SEP) d[k] = q_load(gd + e0 + k * plane);
+        if (!SEP || resume) d[k] = q_load(gd + e0 + k * plane);
       }
     }
   }
@@ -621,7 +649,7 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
     for (int k = 0; k < kn; k++) {
       const uint32_t e = e0 + k * plane;
       if (REG && CM == COEF_PACKED) cs[k * blockDim.x] = *(const uint32_t *)(R.code + e);
-      if (!REG && SEP) q_store(gd + e, zero4);
+      if (!REG && SEP && !resume) q_store(gd + e, zero4);
     }
   }
   // Scalars of the recurrences.  Float sums are scaled by a power of two that
@@ -637,7 +665,8 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
     const double tol = (I.mode == MODE_F32_REFINE ? Sp->itol : I.tol) * Sp->ref_norm;
     S.stop = from_double<T>(tol * tol * scale_t);  // ||r|| < tol as r.r < stop
     S.rz = from_double<T>(Sp->rz_old * scale_t);
-    S.alpha = S.beta = sum_of((T)0);
+    S.alpha = from_double<T>(resume ? Sp->alpha : 0.0);
+    S.beta = from_double<T>(resume ? Sp->beta : 0.0);
   }
   int iter = 0, total = Sp->total_iter, status = Sp->status, phase = PH_INNER;
   const int max_iter = I.max_iter;
@@ -892,9 +921,11 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
       phase = PH_RESID;
       break;
     }
+    if (ROUNDS && iter >= R.budget) break;  // phase INNER
   }
   // hand over to the residual pass: d without the last step, p of the last
-  // step in buffer 0, the scalars
+  // step in buffer 0, the scalars; and z, from which (as from the state after an
+  // update pass) the next launch or phase ticks go on with the inner solve
   if (own) {
 #pragma unroll 1
     for (int k = 0; k < kn; k++) {
@@ -903,20 +934,26 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
       q_store((T *)R.p0 + e0 + k * plane, pv);
     }
     if constexpr (REG) {
+      uint32_t e = opaque(e0);
 #pragma unroll
-      for (int k = 0; k < G; k++)
-        if (k < kn) q_store(gd + e0 + k * plane, d[k]);
+      for (int k = 0; k < G; k++) {
+        if (k < kn) {
+          q_store(gd + e, d[k]);
+          if (ROUNDS && phase == PH_INNER) q_store(gz + e, z[k]);
+        }
+        e += plane;
+      }
     }
   }
   if (cta == 0 && threadIdx.x == 0) {
-    if (phase == PH_RESID) {
+    if (phase != PH_DONE) {
       Sp->alpha = value(S.alpha);
       Sp->beta = value(S.beta);
       Sp->rz_old = value(S.rz) / scale_t;
     }
     if (iter > 0 && isfinite(lead(S.grid[1]))) Sp->relres = sqrt(value(S.grid[1]) / scale_t) / Sp->ref_norm;
     Sp->pbuf = 0;
-    Sp->iter = iter;
+    Sp->iter += iter;  // (0 in the start phase)
     Sp->total_iter = total;
     Sp->status = status;
     Sp->phase = phase;
@@ -1004,7 +1041,8 @@ cudaError_t launch_batch(int build, const Shape &P, const ResWave &R, bool per, 
 }
 
 // Kernel arguments of one grid; threads: of the launch.
-ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &B, void *packets, int slot, int threads) {
+ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &B, void *packets, int slot, int threads,
+                  int budget) {
   ResArgs R;
   R.inst = dI;
   R.packets = packets;
@@ -1034,6 +1072,7 @@ ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &
   R.off_ap = P.off_ap;
   R.off_codes = off_codes(P, I.mode == MODE_F64 ? 8 : 4, threads);
   R.slot = slot;
+  R.budget = budget;
   return R;
 }
 
@@ -1123,7 +1162,7 @@ cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, voi
   if (e != cudaSuccess) return e;
   const bool per = I.periodic != 0;
   ResOne R;
-  R.grid[0] = grid_args(P, I, B.inst, B, packets, 0, P.threads);
+  R.grid[0] = grid_args(P, I, B.inst, B, packets, 0, P.threads, INT_MAX);
   const Shape L{P.ctas, P.threads, smem_of(P, I.mode == MODE_F64 ? 8 : 4, I.coef, P.threads)};
   if (I.mode == MODE_F64) {
     if (I.coef == COEF_F64) return launch_f64<COEF_F64>(L, R, per, st);
@@ -1135,7 +1174,7 @@ cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, voi
 }
 
 cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *const *I, const int *slot,
-                                  const Batch &B, void *packets, size_t packet_bytes, cudaStream_t st) {
+                                  const Batch &B, void *packets, size_t packet_bytes, int budget, cudaStream_t st) {
   const cudaError_t e = cudaMemsetAsync(packets, 0, packet_bytes, st);
   if (e != cudaSuccess) return e;
   Shape L{0, 0, 0};
@@ -1145,7 +1184,7 @@ cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *co
   for (int k = 0; k < n; k++) {
     W.first[k] = L.ctas;
     W.grid[k] = grid_args(*P[k], *I[k], B.inst + slot[k], B, (Packet *)packets + (size_t)2 * PACKET_STRIDE * L.ctas,
-                          slot[k], L.threads);
+                          slot[k], L.threads, budget);
     L.ctas += P[k]->ctas;
     L.smem = std::max(L.smem, smem_of(*P[k], 4, COEF_PACKED, L.threads));
   }

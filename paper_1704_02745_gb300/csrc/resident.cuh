@@ -25,6 +25,7 @@ struct ResArgs {  // kernel arguments
   uint32_t gpr_magic;  // for division by gpr
   int by, bz, nby, nbz, gpr, off_codes, off_ap;
   int slot;            // its place among the batch's instances
+  int budget;          // iterations after which the launch leaves an inner solve in phase INNER
 };
 // The grids of a launch, a run of CTAs each: grid n has CTAs first[n] .. first[n + 1] - 1.
 constexpr int RES_MAX_GRIDS = 16;
@@ -50,9 +51,10 @@ size_t resident_packet_bytes(int ctas);  // of a launch
 bool resident_batch_plan(int nx, int ny, int nz, int num_sms, int max_smem, ResPlan *out);
 // Inner solves of n <= RES_MAX_GRIDS instances of a batch (slot[k], descriptor
 // *I[k] on the host, plans of one build, all periodic or none) that are in
-// their start phase, side by side: at most the plans' room CTAs together.
+// their start phase, or that were left at the budget by an earlier launch, side by
+// side, `budget` iterations of each at most: at most the plans' room CTAs together.
 cudaError_t launch_resident_batch(int n, const ResPlan *const *P, const Inst *const *I, const int *slot,
-                                  const Batch &B, void *packets, size_t packet_bytes, cudaStream_t st);
+                                  const Batch &B, void *packets, size_t packet_bytes, int budget, cudaStream_t st);
 // One inner solve of the batch's only instance (I: its descriptor on the host)
 // if it is in its start phase.
 cudaError_t launch_resident(const ResPlan &P, const Inst &I, const Batch &B, void *packets, size_t packet_bytes,

@@ -601,6 +601,16 @@ Batch server_batch(const pb_server *s) {
 // 133; 32 with wrap of 97x81x113 284 -> 93.  Grids too large for it (some 2.5 M
 // nodes), FP64 and servers created with poll_every > 0 run in ticks.
 
+// Iterations of a grid in a round at most, so that admission, results and
+// cancellations never wait for a slowly converging solve (a launch: 1 to 3 ms).
+// An inner solve that is not done goes on in the next round: always after the same
+// iterations, whatever else runs.  Above the 60 to 140 iterations of ordinary inner
+// solves: 32 of 129^3 (131 each) 168 ms with 128, 166 with 192 and without a limit.
+#ifndef PB_ROUND_ITERS
+#define PB_ROUND_ITERS 192
+#endif
+constexpr int ROUND_ITERS = PB_ROUND_ITERS;
+
 // The residual pass, an inner solve of each grid of `run`, the residual pass.
 // *refused: the device refused a launch; ticks go on from the state as it stands.
 bool run_resident_round(pb_server *s, std::vector<int> run, bool *refused) {
@@ -639,7 +649,7 @@ bool run_resident_round(pb_server *s, std::vector<int> run, bool *refused) {
       P[k] = &s->slots[l.slots[k]].res_plan;
       I[k] = s->slots[l.slots[k]].inst.get();
     }
-    if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, s->stream) != cudaSuccess) {
+    if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, ROUND_ITERS, s->stream) != cudaSuccess) {
       cudaGetLastError();
       *refused = true;
       return true;
