@@ -343,7 +343,8 @@ typedef struct {
  * a grid the device has no memory for (after idle grids are released and the
  * allocation retried once) fails its request with PB_ERR_OOM; a timed-out
  * device wait in a batch fails every solve then on the device with
- * PB_ERR_TIMEOUT (their grids are released). */
+ * PB_ERR_TIMEOUT (their grids are released).  A solve on the chip that waits in
+ * vain for SMs that other work holds is no such failure: it starts over in ticks. */
 pb_status pb_server_create(pb_ctx *ctx, size_t hbm_budget_bytes, const pb_solve_opts *opts,
                            pb_server **out);
 pb_status pb_server_destroy(pb_server *server);

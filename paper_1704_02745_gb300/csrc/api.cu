@@ -1065,7 +1065,7 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
   if (o->profile) {
     if ((st = profiled_loop(g, mode, coef, max_ticks, info))) return st;
   } else {
-    int *herr_poll = (int *)(hs + 1);  // pinned slot after the scalars
+    int *herr_poll = (int *)(hs + 1);  // pinned, after the scalars: two words
     for (;;) {
       if (resident) {
         const cudaError_t e = run_resident(g, I, mode, coef);
@@ -1079,10 +1079,10 @@ extern "C" pb_status pb_pcg_solve(pb_grid *g, const pb_solve_opts *o, double *ph
       if (!resident && (st = pb_run_ticks(g, mode, coef, ticks))) return st;
       done_ticks += resident ? 1 : ticks;  // (a resident graph advances by an inner solve at least)
       CK(cudaMemcpyAsync(hs, g->scal, sizeof(Scal), cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(herr_poll, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-      g->ctx->stats->d2h += sizeof(Scal) + sizeof(int);
+      CK(cudaMemcpyAsync(herr_poll, g->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+      g->ctx->stats->d2h += sizeof(Scal) + 2 * sizeof(int);
       CK(cudaStreamSynchronize(s));
-      if (*herr_poll & ERR_RESIDENT) {
+      if (herr_poll[ERR_RESIDENT]) {
         // The CTAs of an inner solve did not all come to run within its waits' limit (other
         // work held their SMs), and left its vectors in pieces: over again, in ticks.
         if ((st = start())) return st;

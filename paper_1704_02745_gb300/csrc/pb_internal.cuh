@@ -123,13 +123,15 @@ struct Item {  // one unit of work of a phase kernel
   int tile;
 };
 
-// Bits of the error words.
+// An error block (four ints).  Word 0: bits.  Word 1: not 0 once a grid-wide wait of
+// the resident form has given up (phase ticks can do the solve over); a word of its own,
+// cleared without touching what ticks that run meanwhile have to say.
 enum ErrorBit : int {
   ERR_ATOM = 1,        // setup: an atom's trilinear cell leaves the grid
   ERR_WAIT = 2,        // a phase kernel's wait for its loads gave up: the solve cannot finish
   ERR_INTERVALS = 4,   // setup: an edge meets too many spheres
-  ERR_RESIDENT = 8,    // a grid-wide wait of the resident form gave up: phase ticks can solve it
 };
+constexpr int ERR_RESIDENT = 1;  // the word
 
 // Ints of the count block of a batch: [0] stencil items, [1] update items,
 // [2] residual passes pending, [3] unused, [4..9] work counters, [10] the

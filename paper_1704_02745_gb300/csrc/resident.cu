@@ -229,7 +229,7 @@ __device__ __forceinline__ bool await_word(const Packet *words, int c, Sum<T> (&
 #pragma unroll 1
   while (!wire_load(words + (size_t)PACKET_STRIDE * c, x, epoch)) {
     ++polls;
-    if (polls >= RES_MAX_POLLS || ((polls & 255) == 0 && (load_error(err) & ERR_RESIDENT))) return false;
+    if (polls >= RES_MAX_POLLS || ((polls & 255) == 0 && load_error(err) != 0)) return false;
   }
   return true;
 }
@@ -298,7 +298,7 @@ __device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, int cta, int
     }
   }
   if (!ok) {
-    atomicOr(err, ERR_RESIDENT);
+    atomicOr(err, 1);
     S.failed = 1;
   }
   __syncthreads();
@@ -1046,7 +1046,7 @@ ResArgs grid_args(const ResPlan &P, const Inst &I, const Inst *dI, const Batch &
   ResArgs R;
   R.inst = dI;
   R.packets = packets;
-  R.err = B.error;
+  R.err = B.error + ERR_RESIDENT;
   R.resid_pending = B.resid_pending;
   R.resid_list = B.resid_list;
   R.z = I.z;

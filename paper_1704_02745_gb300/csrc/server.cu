@@ -167,7 +167,7 @@ struct Stage {
   Inst *inst = nullptr;   // descriptors of slots [0, MAX_SLOTS)
   Item *items = nullptr;  // stencil items, then update items
   size_t cap_items = 0;
-  int *counts = nullptr;  // 2 ints
+  int *counts = nullptr;  // item counts (2), then the error block's first two words
   int *start = nullptr;   // slots whose solves start
   Scal *scal = nullptr;   // scalars of all slots after the round's graph
   double *energy = nullptr;
@@ -612,13 +612,14 @@ Batch server_batch(const pb_server *s) {
 constexpr int ROUND_ITERS = PB_ROUND_ITERS;
 
 // The residual pass, an inner solve of each grid of `run`, the residual pass.
-// *refused: the device refused a launch; ticks go on from the state as it stands.
-bool run_resident_round(pb_server *s, std::vector<int> run, bool *refused) {
-  *refused = false;
+// *refused: why the device refused a launch, if it did; ticks go on from the state
+// as it stands.
+bool run_resident_round(pb_server *s, std::vector<int> run, cudaError_t *refused) {
+  *refused = cudaSuccess;
   const Batch B = server_batch(s);
   const size_t bytes = resident_packet_bytes(RES_MAX_PER_SM * s->ctx->num_sms);
   if (!s->d_packets && pb_dalloc(&s->d_packets, bytes)) {
-    *refused = true;
+    *refused = cudaErrorMemoryAllocation;
     return true;
   }
   if (!cuda_ok(launch_phase(B, s->mode, s->coef, s->kg, 4, s->stream), s, "residual pass")) return false;
@@ -649,14 +650,39 @@ bool run_resident_round(pb_server *s, std::vector<int> run, bool *refused) {
       P[k] = &s->slots[l.slots[k]].res_plan;
       I[k] = s->slots[l.slots[k]].inst.get();
     }
-    if (launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, ROUND_ITERS, s->stream) != cudaSuccess) {
+    *refused = launch_resident_batch(n, P, I, l.slots.data(), B, s->d_packets, bytes, ROUND_ITERS, s->stream);
+    if (*refused != cudaSuccess) {
       cudaGetLastError();
-      *refused = true;
       return true;
     }
   }
   s->ctx->stats->launches += 2 + launches.size();
   return cuda_ok(launch_phase(B, s->mode, s->coef, s->kg, 4, s->stream), s, "residual pass");
+}
+
+// A grid-wide wait of the last round's resident solves gave up: the CTAs of a launch
+// did not all come to run within the limit, beside other work that held their SMs.
+// The error word does not say which grid's wait it was, so each solve that ran
+// (`run`) starts over in ticks, which wait for no other CTA, from the x it had.
+// Its scalars hold the new start from round `from` on.  at: free entries of sg.start.
+bool restart_in_ticks(pb_server *s, Stage &sg, size_t at, const std::vector<int> &run, uint64_t from) {
+  size_t n = 0;
+  for (int j : run) {
+    Slot &sl = s->slots[j];
+    if (!sl.g || !sl.busy || sl.pending || sl.stopping) continue;
+    sl.ticked = true;
+    sl.first_round = from;
+    sg.start[at + n++] = j;
+  }
+  if (n > 0) {
+    if (!cuda_ok(cudaMemcpyAsync(s->d_list + at, sg.start + at, n * sizeof(int), cudaMemcpyHostToDevice, s->stream),
+                 s, "restart") ||
+        !cuda_ok(launch_start(s->d_inst, s->d_list + at, (int)n, s->d_counts + 2, s->d_rlist, s->stream), s, "restart"))
+      return false;
+    s->ctx->stats->launches += 1;
+    s->ctx->stats->h2d += n * sizeof(int);
+  }
+  return cuda_ok(cudaMemsetAsync(s->d_err + ERR_RESIDENT, 0, sizeof(int), s->stream), s, "clear error");
 }
 
 bool run_graph(pb_server *s, bool stale) {
@@ -940,6 +966,7 @@ void worker_main(pb_server *s) {
   bool active_changed = true, graph_stale = true;
   bool prev_graph = false;             // the previous round ran a graph: its scalars are unread
   std::vector<int> prev_active;        // ... over these slots
+  std::vector<int> prev_run;           // ... of which these ran resident, not yet looked at
   std::vector<Finishing> finishing;    // results queued in the previous round
   std::vector<int> pending;            // admitted, setups not yet seen complete
   while (true) {
@@ -1014,6 +1041,17 @@ void worker_main(pb_server *s) {
     }
     // While kernels are measured every solve runs in the ticks that are measured.
     const bool profiling = s->profiling.load();
+    // Looks at how the last round's resident solves ended, once, before their next launch.
+    auto settle = [&](uint64_t from) -> bool {
+      if (prev_run.empty()) return true;
+      if (!cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) return false;
+      std::vector<int> run;
+      run.swap(prev_run);
+      if (!sp.counts[2 + ERR_RESIDENT]) return true;
+      active_changed = true;
+      return restart_in_ticks(s, sg, started.size(), run, from);
+    };
+    if (profiling && !settle(s->round)) break;
     if (profiling)
       for (Slot &sl : s->slots)
         if (sl.g && sl.busy && !sl.pending && in_resident_form(s, sl)) {
@@ -1066,11 +1104,13 @@ void worker_main(pb_server *s) {
       if (!active.empty() && !rebuild_batch(s, sg, &graph_stale)) break;
     }
     if (want_tune) {
+      if (!settle(s->round)) break;
       for (int j : active) s->slots[j].ticked = true;  // the passes are timed on live solves
       if (!tune_batch(s, sg, active, &graph_stale)) break;
       if (!rebuild_batch(s, sg, &graph_stale)) break;
     }
     bool ran = false;
+    std::vector<int> ran_resident;
     if (!active.empty()) {
       std::vector<int> chip;
       for (int j : active)
@@ -1084,20 +1124,26 @@ void worker_main(pb_server *s) {
       if (!chip.empty()) {
         // what the last round left: grids that finished in it take no SMs
         if (prev_graph && !cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) break;
+        if (!settle(s->round)) break;
         std::vector<int> run;
         for (int j : chip)
-          if (s->slots[j].first_round == s->round || !prev_graph || sp.scal[j].phase != PH_DONE) run.push_back(j);
-        bool refused = false;
+          if (in_resident_form(s, s->slots[j]) &&
+              (s->slots[j].first_round == s->round || !prev_graph || sp.scal[j].phase != PH_DONE))
+            run.push_back(j);
+        cudaError_t refused = cudaSuccess;
         if (!run.empty() && !run_resident_round(s, run, &refused)) break;
-        if (refused) {
-          s->resident_off = true;
+        if (refused != cudaSuccess) {
+          for (int j : run) s->slots[j].ticked = true;
           active_changed = true;
+          // memory may be free again for later solves; any other refusal stands
+          if (refused != cudaErrorMemoryAllocation) s->resident_off = true;
         }
+        ran_resident.swap(run);
       }
       const int hi = *std::max_element(active.begin(), active.end()) + 1;
       cudaMemcpyAsync(sg.scal, s->d_scal, hi * sizeof(Scal), cudaMemcpyDeviceToHost, s->stream);
-      cudaMemcpyAsync(sg.counts + 2, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
-      s->ctx->stats->d2h += hi * sizeof(Scal) + sizeof(int);
+      cudaMemcpyAsync(sg.counts + 2, s->d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+      s->ctx->stats->d2h += hi * sizeof(Scal) + 2 * sizeof(int);
       if (!cuda_ok(cudaEventRecord(sg.ev_graph, s->stream), s, "event")) break;
       ran = true;
     }
@@ -1109,7 +1155,9 @@ void worker_main(pb_server *s) {
     }
     if (prev_graph) {
       if (!cuda_ok(cudaEventSynchronize(sp.ev_graph), s, "round")) break;
-      if (sp.counts[2] & (ERR_WAIT | ERR_RESIDENT)) {
+      // (this round's copy of the scalars is from before a start here: from the next on)
+      if (!settle(s->round + 1)) break;
+      if (sp.counts[2] & ERR_WAIT) {
         // A pipeline wait gave up in that graph (bounded device wait): the
         // grid whose tile was abandoned can no longer finish, and the error
         // word does not say which.  Fail every solve on the device with
@@ -1126,6 +1174,7 @@ void worker_main(pb_server *s) {
         active_changed = true;
         prev_graph = false;
         prev_active.clear();
+        prev_run.clear();
         s->round++;
         continue;
       }
@@ -1144,6 +1193,7 @@ void worker_main(pb_server *s) {
     }
     prev_graph = ran;
     prev_active.swap(active);
+    prev_run.swap(ran_resident);
     s->round++;
   }
   // hand out what was queued, fail what is left
