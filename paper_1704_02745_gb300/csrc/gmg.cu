@@ -252,12 +252,14 @@ template <typename T> __device__ __forceinline__ V4<T> ld4_if(bool in, const T *
   return in ? ld4(p) : V4<T>{};
 }
 // A float as a double without the FP64 pipe (a conversion takes it as long as
-// a multiplication): bits moved, subnormal floats as 0.
+// a multiplication): bits moved; a subnormal float is first scaled by 2^32, exactly.
 __device__ __forceinline__ double widen(float f) {
-  const uint32_t u = __float_as_uint(f), e = u & 0x7F800000u;
-  uint32_t hi = ((u & 0x7FFFFFFFu) >> 3) + 0x38000000u + (e == 0x7F800000u ? 0x38000000u : 0u);
-  hi |= u & 0x80000000u;
-  return e ? __hiloint2double((int)hi, (int)(u << 29)) : 0.0;
+  const bool small = fabsf(f) < 1.17549435e-38f;
+  const uint32_t u = __float_as_uint(small ? f * 4294967296.f : f);
+  uint32_t hi = ((u & 0x7FFFFFFFu) >> 3) + 0x38000000u + ((u & 0x7F800000u) == 0x7F800000u ? 0x38000000u : 0u);
+  hi -= small ? 32u << 20 : 0u;
+  hi = (u & 0x7FFFFFFFu) ? hi : 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
 // {diag, 1 / diag} of the packed operator by code byte.
