@@ -58,10 +58,11 @@ __device__ __forceinline__ double mid_coord(double o, long i, double h) {
 //
 // Bound by FP64 work, which a warp pays for whole when one lane needs it: the box
 // is found in FP32 (nodes too many change nothing), and the margin is tight.
-// The FP32 error of d^2 is below 3e-7 (r + h)^2 + 1e-6 (offsets to 1e-7 of the
-// distance and one rounding each), the margin 50 times that and more.  129^3 with
+// Near the surface an offset is off by u (6 r + 8 h) at most (u = 2^-24: the box's
+// first node, the steps from it, their sum), so d^2 by 1.3e-6 r^2 + 1.7e-6 r h; the
+// margin is twice that and more (the term in h matters where h > 100 r).  129^3 with
 // 2,500 atoms: 107 -> 64 us, 33^3 with 200: 26 -> 18 (FP64 box, margin 1e-3).
-constexpr float INSIDE_MARGIN = 1e-4f;  // relative to r^2 + 1
+constexpr float INSIDE_MARGIN = 1e-4f, STEP_MARGIN = 4e-6f;  // relative to r^2 + 1 and to r h
 // First and last index of the nodes of one axis that lie, or whose edges' midpoints
 // lie, within r of x (x relative to the origin): half a spacing more, and room for
 // the FP32 error of a coordinate of up to n spacings.
@@ -80,7 +81,7 @@ __global__ void k_eps_scatter(const dbl4 *atoms, int n_atoms, Geom g, uint32_t *
   if (a >= n_atoms) return;
   const dbl4 A = atoms[a];  // x, y, z, radius
   const double r2 = __dmul_rn(A.w, A.w);
-  const float r2f = (float)r2, margin = INSIDE_MARGIN * (r2f + 1.0f);
+  const float r2f = (float)r2, margin = INSIDE_MARGIN * (r2f + 1.0f) + STEP_MARGIN * (float)A.w * (float)g.h;
   long i0, i1, j0, j1, k0, k1;
   const float rf = (float)A.w, inv_h = 1.0f / (float)g.h;
   box_axis(A.x - g.ox, rf, inv_h, g.nx, !g.periodic, i0, i1);
