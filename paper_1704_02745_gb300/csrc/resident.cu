@@ -247,8 +247,7 @@ __device__ __forceinline__ bool await_word(const Packet *words, int c, Sum<T> (&
 // publish: what the CTA's threads stored before the call is visible to the
 // neighbours' threads after it: a release fence before the CTA's word, and
 // the last warp waits for the neighbours' words and fences, beside the sum.
-// At least four warps a CTA.  Out of line: the kernel's code is larger than the
-// instruction caches that feed it.
+// At least four warps a CTA.
 template <typename T, int N, int NTH>
 __device__ __forceinline__ bool grid_sum(T v0, T v1, Packet *words, int cta, int ncta, uint32_t epoch, bool publish,
                                          int *err, SumScratch<T, NTH> &S, bool first) {
@@ -669,8 +668,11 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
     const double tol = (I.mode == MODE_F32_REFINE ? Sp->itol : I.tol) * Sp->ref_norm;
     S.stop = from_double<T>(tol * tol * scale_t);  // ||r|| < tol as r.r < stop
     S.rz = from_double<T>(Sp->rz_old * scale_t);
-    S.alpha = from_double<T>(resume ? Sp->alpha : 0.0);
-    S.beta = from_double<T>(resume ? Sp->beta : 0.0);
+    S.alpha = S.beta = sum_of((T)0);
+    if constexpr (ROUNDS) {
+      S.alpha = from_double<T>(resume ? Sp->alpha : 0.0);
+      S.beta = from_double<T>(resume ? Sp->beta : 0.0);
+    }
   }
   int iter = 0, total = Sp->total_iter, status = Sp->status, phase = PH_INNER;
   const int max_iter = I.max_iter;
@@ -950,14 +952,14 @@ __global__ void __launch_bounds__(NTH, ctas_per_sm(NTH)) k_cg_resident(const __g
     }
   }
   if (cta == 0 && threadIdx.x == 0) {
-    if (phase != PH_DONE) {
+    if (ROUNDS ? phase != PH_DONE : phase == PH_RESID) {
       Sp->alpha = value(S.alpha);
       Sp->beta = value(S.beta);
       Sp->rz_old = value(S.rz) / scale_t;
     }
     if (iter > 0 && isfinite(lead(S.grid[1]))) Sp->relres = sqrt(value(S.grid[1]) / scale_t) / Sp->ref_norm;
     Sp->pbuf = 0;
-    Sp->iter += iter;  // (0 in the start phase)
+    Sp->iter = ROUNDS ? Sp->iter + iter : iter;  // (0 in the start phase)
     Sp->total_iter = total;
     Sp->status = status;
     Sp->phase = phase;
