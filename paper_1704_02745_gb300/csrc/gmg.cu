@@ -272,9 +272,11 @@ __device__ __forceinline__ void mg_table(const MgOp &A, float2 *tab) {
 }
 
 // a / b, correctly rounded, from rb = 1 / b correctly rounded: Markstein's
-// correction of a quotient by its exact remainder.
+// correction of a quotient by its exact remainder.  A remainder, or a quotient, that
+// a normal float cannot hold takes the division.
 __device__ __forceinline__ float mg_div(float a, float b, float rb) {
   const float q = a * rb;
+  if (fminf(fabsf(a) * 0x1p-24f, fabsf(q)) < 0x1p-125f && a != 0.f) return __fdiv_rn(a, b);
   return fmaf(fmaf(-q, b, a), rb, q);
 }
 // One damped-Jacobi step of a node: u + (omega (r - A u)) / diag, s the sum of
