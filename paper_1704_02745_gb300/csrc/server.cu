@@ -30,7 +30,9 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <condition_variable>
+#include <cstdint>
 #include <cstring>
 #include <deque>
 #include <memory>
@@ -145,6 +147,7 @@ struct Slot {
   Request req;
   bool warm = false;
   uint64_t first_round = 0;   // round whose graph first runs the current solve
+  uint64_t last_ran = 0;      // last round of its resident form, or the one it joined the batch in
   std::unique_ptr<Inst> inst; // its descriptor, as last uploaded
   ResPlan res_plan;           // plan of its resident inner solves
   bool res_fits = false;      // it has one: its solves run in the resident form
@@ -610,11 +613,19 @@ Batch server_batch(const pb_server *s) {
 #define PB_ROUND_ITERS 192
 #endif
 constexpr int ROUND_ITERS = PB_ROUND_ITERS;
+// Launches of a round that also runs ticks, in turns: one for every 150 M nodes in ticks,
+// one at least (8 iterations of these take 7 ms, 192 of a launch's grids 1 to 3), so that neither the large grids' ticks wait for every small grid nor, under
+// load, the small ones for the large.  Mixed stream, p99 of all / of grids on the chip /
+// of grids in ticks at 80% and 100% of its capacity: so 214 / 153 / 226 and 695 / 685 / 707
+// ms; always one 203 / 152 / 217 and 1,696 / 1,743 / 511; every launch 234 / 175 / 245 and
+// 1,220 / 1,144 / 1,238 (all grids in ticks: 151 and 545, p50 63 ms for 40 at 80%).
+constexpr double LAUNCH_NODES = 150e6;
 
 // The residual pass, an inner solve of each grid of `run`, the residual pass.
 // *refused: why the device refused a launch, if it did; ticks go on from the state
 // as it stands.
-bool run_resident_round(pb_server *s, std::vector<int> run, cudaError_t *refused) {
+// most: launches at most; the grids that have waited longest run, and run becomes theirs.
+bool run_resident_round(pb_server *s, std::vector<int> &run, size_t most, cudaError_t *refused) {
   *refused = cudaSuccess;
   const Batch B = server_batch(s);
   const size_t bytes = resident_packet_bytes(RES_MAX_PER_SM * s->ctx->num_sms);
@@ -626,6 +637,7 @@ bool run_resident_round(pb_server *s, std::vector<int> run, cudaError_t *refused
   // launches: grids of one build, largest first, each into the first with room
   struct Launch {
     int ctas = 0;
+    uint64_t waiting = UINT64_MAX;  // the round since which a grid of it has waited
     std::vector<int> slots;
   };
   auto kind = [&](int j) { return 2 * s->slots[j].res_plan.build + (s->slots[j].g->d.periodic ? 1 : 0); };
@@ -641,7 +653,16 @@ bool run_resident_round(pb_server *s, std::vector<int> run, cudaError_t *refused
     if (it == launches.end()) it = launches.insert(launches.end(), Launch());
     it->ctas += ctas;
     it->slots.push_back(j);
+    it->waiting = std::min(it->waiting, s->slots[j].last_ran);
   }
+  if (launches.size() > most) {
+    std::stable_sort(launches.begin(), launches.end(),
+                     [](const Launch &a, const Launch &b) { return a.waiting < b.waiting; });
+    launches.resize(most);
+    run.clear();
+    for (const Launch &l : launches) run.insert(run.end(), l.slots.begin(), l.slots.end());
+  }
+  for (int j : run) s->slots[j].last_ran = s->round;
   for (const Launch &l : launches) {
     const ResPlan *P[RES_MAX_GRIDS];
     const Inst *I[RES_MAX_GRIDS];
@@ -999,7 +1020,7 @@ void worker_main(pb_server *s) {
       if (q != cudaSuccess) cuda_ok(q, s, "setup");
       s->slots[j].pending = false;
       s->slots[j].ticked = false;
-      s->slots[j].first_round = s->round;
+      s->slots[j].first_round = s->slots[j].last_ran = s->round;
       started.push_back(j);
       pending.erase(pending.begin() + k);
     }
@@ -1131,7 +1152,14 @@ void worker_main(pb_server *s) {
               (s->slots[j].first_round == s->round || !prev_graph || sp.scal[j].phase != PH_DONE))
             run.push_back(j);
         cudaError_t refused = cudaSuccess;
-        if (!run.empty() && !run_resident_round(s, run, &refused)) break;
+        double tick_nodes = 0;
+        for (int j : active) {
+          const pb_grid_desc &d = s->slots[j].g->d;
+          if (!in_resident_form(s, s->slots[j])) tick_nodes += (double)d.nx * d.ny * d.nz;
+        }
+        const size_t most = chip.size() == active.size()
+                                ? SIZE_MAX : (size_t)std::max(1.0, std::round(tick_nodes / LAUNCH_NODES));
+        if (!run.empty() && !run_resident_round(s, run, most, &refused)) break;
         if (refused != cudaSuccess) {
           for (int j : run) s->slots[j].ticked = true;
           active_changed = true;
