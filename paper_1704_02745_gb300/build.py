@@ -73,8 +73,9 @@ FAULT_LIB = os.path.join(FAULT_BUILD, "libpb_faulttest.so")
 
 def build_fault_test(force: bool = False) -> str:
     """A separate copy of the library for the failure-path tests, compiled with
-    -DPB_FAULT_TEST: it adds two test hooks (pb_test_abandon_waits: the next
-    first-plane stage waits give up at once; pb_test_fail_allocs: the next
+    -DPB_FAULT_TEST: it adds three test hooks (pb_test_abandon_waits: the next
+    first-plane stage waits and grid-wide sums give up at once;
+    pb_test_abandon_sums: the next grid-wide sums; pb_test_fail_allocs: the next
     device allocations fail) and is never loaded by the product path."""
     deps = _deps()
     if not force and os.path.exists(FAULT_LIB) and all(

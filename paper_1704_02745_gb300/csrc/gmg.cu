@@ -1230,7 +1230,7 @@ static void vcycle(pb_mg *m, size_t l, cudaStream_t s, unsigned long long &launc
 // kernels after convergence return at once.  Called by pb_pcg_solve for
 // PB_PRECOND_GMG.
 //
-// Measured, an iteration at 33^3 / 129^3 / 257^3: 83 / 218 / 1,100 us.  With
+// Measured, an iteration at 33^3 / 129^3 / 257^3: 83 / 205 / 1,050 us.  With
 // every sweep, transfer, dot product and scalar a kernel of its own, a node a
 // thread (74 launches), and explicit coefficients on every level: 122 / 287 /
 // 1,524 us.  What bounds it now: the FP64 work of the outer CG (13 operations a
